@@ -41,7 +41,7 @@ fdm_status build_group(Dev& d, Arena& A, const fdm_params& p, int count, int gat
     const size_t n = (size_t)p.n1 * p.n2;
     d.geom = geometry<T>(p.n1, p.n2);
     if (d.geom.row_smem > 200 * 1024 || d.geom.col_smem > 200 * 1024) return FDM_ERR_INVALID_ARG;
-    FDM_CK(configure_kernels<T>());
+    FDM_CK(configure_kernels<T>(p.n1, p.n2));
     fdm_status st;
     const size_t cn = (size_t)count * n;
     if ((st = A.alloc(&d.phi[0], cn * sizeof(T)))) return st;
@@ -354,7 +354,7 @@ fdm_status ensure_readout64(fdm_handle* h) {
     r.p = p;
     r.p.precision = FDM_FP64;
     r.count = 1;
-    FDM_CK(configure_kernels<double>());
+    FDM_CK(configure_kernels<double>(p.n1, p.n2));
     r.geom = geometry<double>(p.n1, p.n2);
     const size_t n = h->n;
     if ((st = h->arena.alloc(&r.spec, n * sizeof(double)))) return st;

@@ -75,7 +75,7 @@ template <typename T> void knp_shape_info(int shape, int* ty, int* npt, int* min
 template <typename T> cudaError_t autotune_group(Dev& d, cudaStream_t s);
 // fill U13 (buffer 0 of every instance) with a smooth synthetic field with kinks
 template <typename T> void launch_tune_fill(const Dev& d, cudaStream_t s);
-template <typename T> cudaError_t configure_kernels();
+template <typename T> cudaError_t configure_kernels(int n1, int n2);
 // step launches read U13 from phi[sc[i].cur] of every instance and write the other buffer
 template <typename T> void launch_step(const Dev& d, cudaStream_t s);
 template <typename T> void launch_phase(const Dev& d, int phase, cudaStream_t s);

@@ -14,78 +14,9 @@
 // multiply by K, inverse FFT along x2) -> row_inverse (C2R, tau and max|v0|) -> knp_step.
 #include <type_traits>
 
-#include "fdm_device.cuh"
-#include "fdm_internal.h"
+#include "fdm_step.cuh"
 
 namespace fdm {
-
-// ------------------------------------------------------------------ small helpers
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-// block-wide sum, fixed order (deterministic); result valid in thread 0
-__device__ double block_sum(double v, double* red) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    __syncthreads();
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0) for (int i = 0; i < nw; ++i) r += red[i];
-    __syncthreads();
-    return r;
-}
-// max of non-negative values, NaN-propagating through the bit order (NaN > +inf)
-__device__ __forceinline__ unsigned long long abs_bits(double v) {
-    return (unsigned long long)__double_as_longlong(fabs(v));
-}
-
-__device__ __forceinline__ void loading_state(const fdm_params& p, long long step, double t, double mean,
-                                              double* eps, double* sig) {
-    const double mu = p.E / (2.0 * (1.0 + p.nu));
-    const double frac = (double)p.nh / (double)p.nz;
-    if (p.loading_mode == FDM_LOAD_STRESS) {
-        *sig = p.sigma_bar13;
-        *eps = (p.sigma_bar13 + mu * frac * mean) / (2.0 * mu);
-    } else if (p.loading_mode == FDM_LOAD_STRAIN_RAMP || p.loading_mode == FDM_LOAD_STRAIN_RATE) {
-        *eps = p.eps_bar13_0 + p.eps_bar13_rate * (p.loading_mode == FDM_LOAD_STRAIN_RAMP ? (double)step : t);
-        *sig = 2.0 * mu * (*eps) - mu * frac * mean;
-    } else {
-        *eps = 0.5 * frac * mean;
-        *sig = 0.0;
-    }
-}
-
-
-// Instance addressing of the step kernels: a launch covers `count` instances (grid y, or z
-// for the stencil).  sc == nullptr marks a set-up launch (one instance, buffer 0, always
-// runs).  Otherwise instance i reads U13 from buffer sc[i].cur, and with gating on it runs
-// only while its step budget sc[i].steps_left is non-zero.  Read by thread 0 only and
-// broadcast, so that every thread of a block sees the same values.
-struct InstCtl {
-    fdm_dev_scalars* sc;
-    int gated;
-};
-
-__device__ __forceinline__ void inst_state(const InstCtl& c, int inst, int* run, int* cur) {
-    int r = 1, k = 0;
-    if (c.sc) {
-        const fdm_dev_scalars* si = c.sc + inst;
-        k = si->cur;
-        if (c.gated && si->steps_left == 0) r = 0;
-    }
-    *run = r;
-    *cur = k;
-}
-
-// Neumaier step s + x with compensation c (FP64; the magnitude test on bit patterns)
-__device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
-    const double t = s + x;
-    c += ((ubits(s) & kMagBits) >= (ubits(x) & kMagBits)) ? (s - t) + x : (x - t) + s;
-    s = t;
-}
 
 // one element global -> shared without passing through registers (4, 8 or 16 bytes)
 template <typename T> __device__ __forceinline__ void copy_async(T* smem_dst, const T* gmem_src) {
@@ -213,66 +144,6 @@ __global__ void __launch_bounds__(FftBounds<T>::threads, FftBounds<T>::minb) row
 
 // ------------------------------------------------------------------ column pass
 // grid: (n1/2) / C blocks; block handles columns [b C, b C + C) of the transposed spectrum.
-// Multiplier modes (all include the 1/(n1 n2) normalisation):
-//   COL_K         tau-hat = K U-hat, DC = sigma_bar13 (block 0 computes <U13> and loading)
-//   COL_DERIV1    alpha12-hat = i xi1 U-hat  (odd symbol, 0 at the x1 Nyquist index)
-//   COL_DERIV2N   alpha11-hat = -i xi2 U-hat (odd symbol, 0 at the x2 Nyquist index)
-//   COL_FWD       forward transform only (no normalisation)
-//   COL_INV       inverse transform only
-//   COL_SYM       stress component on a plane of the 3-D cell: the quarter table Kh holds
-//                 |symbol| for kx, ky >= 0 (normalisation folded in); the symbol is i times
-//                 it when sym_imag, and changes sign with ky when sym_odd2 (the sign in kx
-//                 never enters: kx >= 0 in the half spectrum); DC is zero
-constexpr int kRedLanes = 256;  // lanes of the <U13> reduction in the column kernel
-enum ColMode { COL_K = 0, COL_DERIV1 = 1, COL_DERIV2N = 2, COL_FWD = 3, COL_INV = 4, COL_SYM = 5 };
-
-template <typename T>
-struct ColArgs {
-    fdm_params p;
-    int mode;
-    const double* row_partials;  // COL_K: per-row sums of U13 (nparts = n2 entries)
-    int nparts;
-    fdm_dev_scalars* sc;         // COL_K: scalars of instance 0 (block 0 writes mean/eps/sigma)
-    int gated;                   // COL_K: honour the instances' step budgets
-    T scl;                       // 1 / (n1 n2)
-    T xi1_unit, xi2_unit;        // 2 pi / (n dx): xi = k~ * unit
-    int sym_odd2, sym_imag;      // COL_SYM: symbol odd in xi2; symbol imaginary
-};
-
-template <typename T>
-__device__ __forceinline__ cpx<T> col_multiplier(const ColArgs<T>& a, const T* __restrict__ Kh, int kxi,
-                                                 int ky, int n1, int n2) {
-    // kxi in [0, n1/2]; ky in [0, n2)
-    if (a.mode == COL_K) {   // the table carries the 1/(n1 n2) normalisation
-        int kyf = ky <= n2 / 2 ? ky : n2 - ky;
-        return mk(Kh[(size_t)kxi * (n2 / 2 + 1) + kyf], T(0));
-    }
-    if (a.mode == COL_SYM) {
-        int kyf = ky <= n2 / 2 ? ky : n2 - ky;
-        T v = Kh[(size_t)kxi * (n2 / 2 + 1) + kyf];
-        if (a.sym_odd2 && ky > n2 / 2) v = -v;
-        return a.sym_imag ? mk(T(0), v) : mk(v, T(0));
-    }
-    if (a.mode == COL_DERIV1) {
-        if (2 * kxi == n1) return mk(T(0), T(0));
-        return mk(T(0), T(kxi) * a.xi1_unit * a.scl);
-    }
-    // COL_DERIV2N
-    if (2 * ky == n2) return mk(T(0), T(0));
-    int kys = ky <= n2 / 2 ? ky : ky - n2;
-    return mk(T(0), -(T(kys) * a.xi2_unit) * a.scl);
-}
-
-// the symbol applied to one coefficient: real (K) or imaginary (derivatives), so two
-// multiplications rather than a general complex product
-template <typename T>
-__device__ __forceinline__ cpx<T> col_apply(const ColArgs<T>& a, const T* __restrict__ Kh, int kxi, int ky,
-                                            int n1, int n2, cpx<T> z) {
-    const cpx<T> m = col_multiplier<T>(a, Kh, kxi, ky, n1, n2);
-    if (a.mode == COL_K || (a.mode == COL_SYM && !a.sym_imag)) return mk(m.x * z.x, m.x * z.y);
-    return mk(-(m.y * z.y), m.y * z.x);
-}
-
 // body of one block: columns [tile C, tile C + C) of instance inst
 template <typename T>
 __device__ __forceinline__ void col_pass_body(const cpx<T>* in, cpx<T>* out, int n1, int n2, int C,
@@ -387,62 +258,6 @@ __global__ void __launch_bounds__(FftBounds<T>::threads, FftBounds<T>::minb) col
 // ------------------------------------------------------------------ row inverse (C2R)
 // grid: n2 / R blocks.  mode ROW_PLAIN: write the real rows (+ offset).  ROW_TAU: write
 // tau13 and reduce max |v0| of the celerity law into sc->vmax_bits.
-enum RowMode { ROW_PLAIN = 0, ROW_TAU = 1 };
-
-// celerity law (Sec. 3.2.3 Hamiltonian; Sec. 4.1 prescribed), parameters in the field type
-template <typename T>
-struct VelLaw {
-    int mode;            // FDM_V_PRESCRIBED or FDM_V_STRESS
-    int friction;        // tau_y != 0 and stress driven
-    T v0, mobility;
-    double tau_y, beta;  // lattice friction (FP64; evaluated only when friction != 0)
-    const T* mfac;       // per-cell mobility factor m(x) (heterogeneous drag, Sec. 5.3), or null
-};
-
-template <typename T> VelLaw<T> make_vel(const fdm_params& p, const void* mfac = nullptr) {
-    VelLaw<T> v;
-    v.mfac = static_cast<const T*>(mfac);
-    v.mode = p.velocity_mode;
-    v.friction = (p.tau_y != 0.0 && p.velocity_mode == FDM_V_STRESS) ? 1 : 0;
-    v.v0 = T(p.v0);
-    v.mobility = T(p.mobility);
-    v.tau_y = p.tau_y;
-    v.beta = p.beta;
-    return v;
-}
-
-template <typename T>
-__device__ __forceinline__ T celerity(const VelLaw<T>& v, T tau, T up, double phi_ref) {
-    if (v.mode == FDM_V_PRESCRIBED) return v.v0;
-    if (!v.friction) return -(v.mobility * tau);
-    const T fr = T(v.tau_y * cos(((double)up + phi_ref) / v.beta));
-    return v.mobility * (fr - tau);
-}
-
-// dt from the CFL rule |v0|max dt / dx = CFL (Sec. 4.3, Sec. 5.2), in FP64
-__device__ __forceinline__ double cfl_dt(double vmax, double cfl, double dx, double dt_max) {
-    double dtd;
-    if (vmax > 0.0) {
-        dtd = cfl * dx / vmax;
-        if (dt_max > 0.0 && dtd > dt_max) dtd = dt_max;
-    } else {
-        dtd = dt_max > 0.0 ? dt_max : 0.0;
-    }
-    return dtd;
-}
-
-template <typename T>
-struct RowArgs {
-    VelLaw<T> vel;
-    int mode;
-    const void* phi0;          // ROW_TAU: the two state buffers (U13 is needed for friction)
-    const void* phi1;
-    fdm_dev_scalars* sc;       // ROW_TAU: scalars of instance 0
-    int gated;
-    T offset;                  // ROW_PLAIN: added to every output value
-    double cfl, dx, dt_max;    // ROW_TAU: time-step rule (FP64)
-};
-
 // body of one block: rows [tile R, tile R + R) of instance inst; ntiles = row blocks per
 // instance (the last of them to finish computes the step's dt)
 template <typename T>
@@ -486,7 +301,6 @@ __device__ __forceinline__ void row_inverse_body(const cpx<T>* spec, T* dst, int
     const cpx<T>* z = block_fft<+1>(A, B, L, R, ld, ptw);
     T vmax = T(0);
     bool bad = false;
-    unsigned long long vbits = 0ull;  // FP64: max of |v0| as magnitude bits (a NaN wins)
     const T* up = reinterpret_cast<const T*>(s_cur ? a.phi1 : a.phi0);
     if (up) up += inst * nn;
     const double phi_ref = (sci && a.vel.friction) ? sci->phi_ref : 0.0;
@@ -505,14 +319,8 @@ __device__ __forceinline__ void row_inverse_body(const cpx<T>* spec, T* dst, int
                 c0 = c0 * mf.x;
                 c1 = c1 * mf.y;
             }
-            if constexpr (std::is_same<T, double>::value) {
-                const unsigned long long m0 = ubits(c0) & kMagBits, m1 = ubits(c1) & kMagBits;
-                vbits = m0 > vbits ? m0 : vbits;
-                vbits = m1 > vbits ? m1 : vbits;
-            } else {
-                vmax = tmax(vmax, tmax(tabs(c0), tabs(c1)));
-                bad |= (c0 != c0) || (c1 != c1);
-            }
+            vmax = tmax(vmax, tmax(tabs(c0), tabs(c1)));
+            bad |= (c0 != c0) || (c1 != c1);
             *reinterpret_cast<cpx<T>*>(dst + o) = v;
         } else {
             *reinterpret_cast<cpx<T>*>(dst + o) = mk(v.x + a.offset, v.y + a.offset);
@@ -520,28 +328,8 @@ __device__ __forceinline__ void row_inverse_body(const cpx<T>* spec, T* dst, int
     }
     if (a.mode == ROW_TAU) {
         // NaN-aware block max through the bit pattern of |v| (max is exact in any precision)
-        unsigned long long bits = vbits;
-        if constexpr (!std::is_same<T, double>::value) bits = bad ? 0x7ff8000000000000ull : abs_bits((double)vmax);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            unsigned long long other = __shfl_xor_sync(0xffffffffu, bits, o);
-            bits = other > bits ? other : bits;
-        }
-        if ((threadIdx.x & 31) == 0) atomicMax(&sci->vmax_bits, bits);
-        // the last block of the instance to finish turns max |v0| into this step's dt, once
-        // (every block's maxima are in before its fenced counter increment)
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(&sci->ri_count, 1u) == (unsigned)ntiles - 1u) {
-                __threadfence();
-                const double vmax = __longlong_as_double((long long)atomicAdd(&sci->vmax_bits, 0ull));
-                const double dtd = cfl_dt(vmax, a.cfl, a.dx, a.dt_max);
-                sci->dt_next = dtd;
-                sci->dt_h_next = dtd / a.dx;   // the stencil works in cell units
-                sci->ri_count = 0u;
-            }
-        }
+        step_dt_from_max(bad ? 0x7ff8000000000000ull : abs_bits((double)vmax), sci, (unsigned)ntiles, a.cfl, a.dx,
+                         a.dt_max);
     }
 }
 
@@ -578,24 +366,7 @@ __global__ void celerity_dt_kernel(const T* __restrict__ tau, const T* phi0, con
     }
     unsigned long long bits = vbits;
     if constexpr (!std::is_same<T, double>::value) bits = bad ? 0x7ff8000000000000ull : abs_bits((double)vmax);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long other = __shfl_xor_sync(0xffffffffu, bits, o);
-        bits = other > bits ? other : bits;
-    }
-    if ((threadIdx.x & 31) == 0) atomicMax(&sc->vmax_bits, bits);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(&sc->ri_count, 1u) == gridDim.x - 1) {
-            __threadfence();
-            const double vm = __longlong_as_double((long long)atomicAdd(&sc->vmax_bits, 0ull));
-            const double dtd = cfl_dt(vm, cfl, dx, dt_max);
-            sc->dt_next = dtd;
-            sc->dt_h_next = dtd / dx;
-            sc->ri_count = 0u;
-        }
-    }
+    step_dt_from_max(bits, sc, gridDim.x, cfl, dx, dt_max);
 }
 
 // ------------------------------------------------------------------ KNP stencil
@@ -1117,28 +888,36 @@ void launch_tune_fill(const Dev& d, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t configure_kernels() {
-    // the FFT kernels live on shared memory: allow large dynamic allocations and ask for the
-    // largest shared-memory carveout so that several blocks stay resident per SM
-    const void* fns[3] = {(const void*)row_forward_kernel<T>, (const void*)row_inverse_kernel<T>,
-                          (const void*)col_pass_kernel<T>};
-    for (const void* f : fns) {
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
+cudaError_t configure_kernels(int n1, int n2) {
+    if constexpr (std::is_same<T, double>::value) {
+        return fix_configure(n1, n2);
+    } else {
+        // the FFT kernels live on shared memory: allow large dynamic allocations and ask for the
+        // largest shared-memory carveout so that several blocks stay resident per SM
+        const void* fns[3] = {(const void*)row_forward_kernel<T>, (const void*)row_inverse_kernel<T>,
+                              (const void*)col_pass_kernel<T>};
+        for (const void* f : fns) {
+            cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem);
+            if (e != cudaSuccess) return e;
+            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
     }
-    return cudaSuccess;
 }
 
 template <typename T>
 void launch_row_forward(const Dev& d, const T* src0, const T* src1, cpx<T>* spec, double* partials, InstCtl ctl,
                         int count, cudaStream_t s) {
-    const LaunchGeom& g = d.geom;
-    dim3 grid(g.row_blocks, count);
-    row_forward_kernel<T><<<grid, g.row_threads, g.row_smem, s>>>(src0, src1, spec, d.p.n1, d.p.n2, g.R,
-                                                                (const cpx<T>*)d.tw1, (const cpx<T>*)d.pt1,
-                                                                partials, ctl);
+    if constexpr (std::is_same<T, double>::value) {
+        fix_row_forward(d, src0, src1, spec, partials, ctl, count, s);
+    } else {
+        const LaunchGeom& g = d.geom;
+        dim3 grid(g.row_blocks, count);
+        row_forward_kernel<T><<<grid, g.row_threads, g.row_smem, s>>>(src0, src1, spec, d.p.n1, d.p.n2, g.R,
+                                                                    (const cpx<T>*)d.tw1, (const cpx<T>*)d.pt1,
+                                                                    partials, ctl);
+    }
 }
 
 template <typename T>
@@ -1160,15 +939,19 @@ ColArgs<T> col_args(const Dev& d, int mode, bool with_mean, int sym_odd2 = 0, in
 template <typename T>
 void launch_col(const Dev& d, const cpx<T>* in, cpx<T>* out, int mode, bool with_mean, int count, cudaStream_t s,
                 int sym_odd2 = 0, int sym_imag = 0) {
-    const LaunchGeom& g = d.geom;
-    dim3 grid(g.col_blocks, count);
-    col_pass_kernel<T><<<grid, g.col_threads, g.col_smem, s>>>(in, out, d.p.n1, d.p.n2, g.C, (const cpx<T>*)d.pt2,
-                                                             (const T*)d.Kh,
-                                                             col_args<T>(d, mode, with_mean, sym_odd2, sym_imag));
+    if constexpr (std::is_same<T, double>::value) {
+        fix_col(d, in, out, col_args<T>(d, mode, with_mean, sym_odd2, sym_imag), count, s);
+    } else {
+        const LaunchGeom& g = d.geom;
+        dim3 grid(g.col_blocks, count);
+        col_pass_kernel<T><<<grid, g.col_threads, g.col_smem, s>>>(in, out, d.p.n1, d.p.n2, g.C, (const cpx<T>*)d.pt2,
+                                                                 (const T*)d.Kh,
+                                                                 col_args<T>(d, mode, with_mean, sym_odd2, sym_imag));
+    }
 }
 
 template <typename T>
-RowArgs<T> row_args(const Dev& d, int mode, double offset) {
+RowArgs<T> row_args(const Dev& d, int mode, double offset, bool after_k = false) {
     RowArgs<T> a;
     a.vel = make_vel<T>(d.p, d.mfac);
     a.mode = mode;
@@ -1176,6 +959,7 @@ RowArgs<T> row_args(const Dev& d, int mode, double offset) {
     a.phi1 = d.phi[1];
     a.sc = d.sc;
     a.gated = d.gated;
+    a.add_sigma = after_k ? 1 : 0;
     a.offset = T(offset);
     a.cfl = d.p.cfl;
     a.dx = d.p.dx;
@@ -1184,12 +968,16 @@ RowArgs<T> row_args(const Dev& d, int mode, double offset) {
 }
 template <typename T>
 void launch_row_inverse(const Dev& d, const cpx<T>* spec, T* dst, int mode, double offset, int count,
-                        cudaStream_t s) {
-    const LaunchGeom& g = d.geom;
-    dim3 grid(g.row_blocks, count);
-    row_inverse_kernel<T><<<grid, g.row_threads, g.row_smem, s>>>(spec, dst, d.p.n1, d.p.n2, g.R,
-                                                                (const cpx<T>*)d.tw1, (const cpx<T>*)d.pt1,
-                                                                row_args<T>(d, mode, offset));
+                        cudaStream_t s, bool after_k = false) {
+    if constexpr (std::is_same<T, double>::value) {
+        fix_row_inverse(d, spec, dst, row_args<T>(d, mode, offset, after_k), count, s);
+    } else {
+        const LaunchGeom& g = d.geom;
+        dim3 grid(g.row_blocks, count);
+        row_inverse_kernel<T><<<grid, g.row_threads, g.row_smem, s>>>(spec, dst, d.p.n1, d.p.n2, g.R,
+                                                                    (const cpx<T>*)d.tw1, (const cpx<T>*)d.pt1,
+                                                                    row_args<T>(d, mode, offset));
+    }
 }
 
 template <typename T, int V>
@@ -1236,7 +1024,7 @@ void launch_phase(const Dev& d, int phase, cudaStream_t s) {
     switch (phase) {
         case 0: launch_row_forward<T>(d, (const T*)d.phi[0], (const T*)d.phi[1], spec, d.row_partials, ctl, d.count, s); break;
         case 1: launch_col<T>(d, spec, spec, COL_K, true, d.count, s); break;
-        case 2: launch_row_inverse<T>(d, spec, (T*)d.tau, ROW_TAU, 0.0, d.count, s); break;
+        case 2: launch_row_inverse<T>(d, spec, (T*)d.tau, ROW_TAU, 0.0, d.count, s, true); break;
         default: launch_knp<T>(d, s); break;
     }
 }
@@ -1253,7 +1041,7 @@ template <typename T>
 void launch_static_to(const Dev& d, T* dst, cudaStream_t s) {
     launch_phase<T>(d, 0, s);
     launch_phase<T>(d, 1, s);
-    launch_row_inverse<T>(d, (const cpx<T>*)d.spec, dst, ROW_PLAIN, 0.0, 1, s);
+    launch_row_inverse<T>(d, (const cpx<T>*)d.spec, dst, ROW_PLAIN, 0.0, 1, s, true);
 }
 
 // one stress component of the current state (single instance) with the plane table d.Kh of
@@ -1375,7 +1163,8 @@ __global__ void twiddle_tables_kernel(cpx<T>* __restrict__ tw, int n, cpx<T>* __
     }
 }
 template <typename T> void launch_twiddle_tables(void* tw, int n, void* pt, int L, cudaStream_t s) {
-    twiddle_tables_kernel<T><<<8, 256, 0, s>>>((cpx<T>*)tw, n, (cpx<T>*)pt, L);
+    if constexpr (std::is_same<T, double>::value) fix_tables(tw, n, pt, L, s);
+    else twiddle_tables_kernel<T><<<8, 256, 0, s>>>((cpx<T>*)tw, n, (cpx<T>*)pt, L);
 }
 
 // layer weights |chi-hat(k3)|^2 = sin^2(pi k3 nh / nz) / sin^2(pi k3 / nz) for k3 in
@@ -1608,7 +1397,7 @@ cudaError_t persist_launch(const void* dev_desc, int ngroups, int nsteps, Persis
     template int col_candidates<T>(int, int, int*, int);                                                    \
     template void knp_shape_info<T>(int, int*, int*, int*);                                                 \
     template void launch_tune_fill<T>(const Dev&, cudaStream_t);                                            \
-    template cudaError_t configure_kernels<T>();                                                            \
+    template cudaError_t configure_kernels<T>(int, int);                                                       \
     template void launch_step<T>(const Dev&, cudaStream_t);                                                 \
     template void launch_phase<T>(const Dev&, int, cudaStream_t);                                           \
     template void launch_static<T>(const Dev&, cudaStream_t);                                               \

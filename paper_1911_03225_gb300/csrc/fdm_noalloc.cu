@@ -9,8 +9,7 @@
 #include <cmath>
 #include <mutex>
 
-#include "fdm_device.cuh"
-#include "fdm_internal.h"
+#include "fdm_step.cuh"
 
 namespace fdm {
 namespace {
@@ -43,8 +42,8 @@ bool g_ready[kMaxDevices] = {};
 
 bool pow2_between(int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; }
 
-// Once per device, with that device current: resolve the scratch address and set the
-// kernels' shared-memory limits.
+// Once per device, with that device current: resolve the scratch address and load
+// the kernels.
 fdm_status setup_device(int dev, double** out) {
     std::lock_guard<std::mutex> lock(g_setup_mutex);
     if (!g_ready[dev]) {
@@ -54,7 +53,7 @@ fdm_status setup_device(int dev, double** out) {
         void* ptr = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
         if (e == cudaSuccess && ptr == nullptr) e = cudaErrorInvalidSymbol;
-        if (e == cudaSuccess) e = configure_kernels<double>();
+        if (e == cudaSuccess) e = fix_preload(kMaxSide);   // later calls load nothing, whatever their grid
         if (e != cudaSuccess) {
             cudaGetLastError();
             return e == cudaErrorMemoryAllocation ? FDM_ERR_OOM : FDM_ERR_DEVICE;

@@ -1,0 +1,231 @@
+// fdm_step.cuh -- pieces of the step that its kernels share: instance addressing, the loading
+// law, the column pass's symbols, the celerity law and the time-step rule.
+#pragma once
+#include "fdm_device.cuh"
+#include "fdm_internal.h"
+
+namespace fdm {
+
+// ------------------------------------------------------------------ small helpers
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// block-wide sum, fixed order (deterministic); result valid in thread 0
+__device__ __forceinline__ double block_sum(double v, double* red) {
+    v = warp_sum(v);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    __syncthreads();
+    if (lane == 0) red[w] = v;
+    __syncthreads();
+    double r = 0.0;
+    if (threadIdx.x == 0) for (int i = 0; i < nw; ++i) r += red[i];
+    __syncthreads();
+    return r;
+}
+// max of non-negative values, NaN-propagating through the bit order (NaN > +inf)
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    return (unsigned long long)__double_as_longlong(fabs(v));
+}
+
+__device__ __forceinline__ void loading_state(const fdm_params& p, long long step, double t, double mean,
+                                              double* eps, double* sig) {
+    const double mu = p.E / (2.0 * (1.0 + p.nu));
+    const double frac = (double)p.nh / (double)p.nz;
+    if (p.loading_mode == FDM_LOAD_STRESS) {
+        *sig = p.sigma_bar13;
+        *eps = (p.sigma_bar13 + mu * frac * mean) / (2.0 * mu);
+    } else if (p.loading_mode == FDM_LOAD_STRAIN_RAMP || p.loading_mode == FDM_LOAD_STRAIN_RATE) {
+        *eps = p.eps_bar13_0 + p.eps_bar13_rate * (p.loading_mode == FDM_LOAD_STRAIN_RAMP ? (double)step : t);
+        *sig = 2.0 * mu * (*eps) - mu * frac * mean;
+    } else {
+        *eps = 0.5 * frac * mean;
+        *sig = 0.0;
+    }
+}
+
+
+// Instance addressing of the step kernels: a launch covers `count` instances (grid y, or z
+// for the stencil).  sc == nullptr marks a set-up launch (one instance, buffer 0, always
+// runs).  Otherwise instance i reads U13 from buffer sc[i].cur, and with gating on it runs
+// only while its step budget sc[i].steps_left is non-zero.  Read by thread 0 only and
+// broadcast, so that every thread of a block sees the same values.
+struct InstCtl {
+    fdm_dev_scalars* sc;
+    int gated;
+};
+
+__device__ __forceinline__ void inst_state(const InstCtl& c, int inst, int* run, int* cur) {
+    int r = 1, k = 0;
+    if (c.sc) {
+        const fdm_dev_scalars* si = c.sc + inst;
+        k = si->cur;
+        if (c.gated && si->steps_left == 0) r = 0;
+    }
+    *run = r;
+    *cur = k;
+}
+
+// Neumaier step s + x with compensation c (FP64; the magnitude test on bit patterns)
+__device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
+    const double t = s + x;
+    c += ((ubits(s) & kMagBits) >= (ubits(x) & kMagBits)) ? (s - t) + x : (x - t) + s;
+    s = t;
+}
+
+// Multiplier modes (all include the 1/(n1 n2) normalisation):
+//   COL_K         tau-hat = K U-hat, DC = sigma_bar13 (block 0 computes <U13> and loading)
+//   COL_DERIV1    alpha12-hat = i xi1 U-hat  (odd symbol, 0 at the x1 Nyquist index)
+//   COL_DERIV2N   alpha11-hat = -i xi2 U-hat (odd symbol, 0 at the x2 Nyquist index)
+//   COL_FWD       forward transform only (no normalisation)
+//   COL_INV       inverse transform only
+//   COL_SYM       stress component on a plane of the 3-D cell: the quarter table Kh holds
+//                 |symbol| for kx, ky >= 0 (normalisation folded in); the symbol is i times
+//                 it when sym_imag, and changes sign with ky when sym_odd2 (the sign in kx
+//                 never enters: kx >= 0 in the half spectrum); DC is zero
+constexpr int kRedLanes = 256;  // lanes of the <U13> reduction in the column kernel
+enum ColMode { COL_K = 0, COL_DERIV1 = 1, COL_DERIV2N = 2, COL_FWD = 3, COL_INV = 4, COL_SYM = 5 };
+
+template <typename T>
+struct ColArgs {
+    fdm_params p;
+    int mode;
+    const double* row_partials;  // COL_K: per-row sums of U13 (nparts = n2 entries)
+    int nparts;
+    fdm_dev_scalars* sc;         // COL_K: scalars of instance 0 (block 0 writes mean/eps/sigma)
+    int gated;                   // COL_K: honour the instances' step budgets
+    T scl;                       // 1 / (n1 n2)
+    T xi1_unit, xi2_unit;        // 2 pi / (n dx): xi = k~ * unit
+    int sym_odd2, sym_imag;      // COL_SYM: symbol odd in xi2; symbol imaginary
+};
+
+template <typename T>
+__device__ __forceinline__ cpx<T> col_multiplier(const ColArgs<T>& a, const T* __restrict__ Kh, int kxi,
+                                                 int ky, int n1, int n2) {
+    // kxi in [0, n1/2]; ky in [0, n2)
+    if (a.mode == COL_K) {   // the table carries the 1/(n1 n2) normalisation
+        int kyf = ky <= n2 / 2 ? ky : n2 - ky;
+        return mk(Kh[(size_t)kxi * (n2 / 2 + 1) + kyf], T(0));
+    }
+    if (a.mode == COL_SYM) {
+        int kyf = ky <= n2 / 2 ? ky : n2 - ky;
+        T v = Kh[(size_t)kxi * (n2 / 2 + 1) + kyf];
+        if (a.sym_odd2 && ky > n2 / 2) v = -v;
+        return a.sym_imag ? mk(T(0), v) : mk(v, T(0));
+    }
+    if (a.mode == COL_DERIV1) {
+        if (2 * kxi == n1) return mk(T(0), T(0));
+        return mk(T(0), T(kxi) * a.xi1_unit * a.scl);
+    }
+    // COL_DERIV2N
+    if (2 * ky == n2) return mk(T(0), T(0));
+    int kys = ky <= n2 / 2 ? ky : ky - n2;
+    return mk(T(0), -(T(kys) * a.xi2_unit) * a.scl);
+}
+
+// the symbol applied to one coefficient: real (K) or imaginary (derivatives), so two
+// multiplications rather than a general complex product
+template <typename T>
+__device__ __forceinline__ cpx<T> col_apply(const ColArgs<T>& a, const T* __restrict__ Kh, int kxi, int ky,
+                                            int n1, int n2, cpx<T> z) {
+    const cpx<T> m = col_multiplier<T>(a, Kh, kxi, ky, n1, n2);
+    if (a.mode == COL_K || (a.mode == COL_SYM && !a.sym_imag)) return mk(m.x * z.x, m.x * z.y);
+    return mk(-(m.y * z.y), m.y * z.x);
+}
+
+enum RowMode { ROW_PLAIN = 0, ROW_TAU = 1 };
+
+// celerity law (Sec. 3.2.3 Hamiltonian; Sec. 4.1 prescribed), parameters in the field type
+template <typename T>
+struct VelLaw {
+    int mode;            // FDM_V_PRESCRIBED or FDM_V_STRESS
+    int friction;        // tau_y != 0 and stress driven
+    T v0, mobility;
+    double tau_y, beta;  // lattice friction (FP64; evaluated only when friction != 0)
+    const T* mfac;       // per-cell mobility factor m(x) (heterogeneous drag, Sec. 5.3), or null
+};
+
+template <typename T> VelLaw<T> make_vel(const fdm_params& p, const void* mfac = nullptr) {
+    VelLaw<T> v;
+    v.mfac = static_cast<const T*>(mfac);
+    v.mode = p.velocity_mode;
+    v.friction = (p.tau_y != 0.0 && p.velocity_mode == FDM_V_STRESS) ? 1 : 0;
+    v.v0 = T(p.v0);
+    v.mobility = T(p.mobility);
+    v.tau_y = p.tau_y;
+    v.beta = p.beta;
+    return v;
+}
+
+template <typename T>
+__device__ __forceinline__ T celerity(const VelLaw<T>& v, T tau, T up, double phi_ref) {
+    if (v.mode == FDM_V_PRESCRIBED) return v.v0;
+    if (!v.friction) return -(v.mobility * tau);
+    const T fr = T(v.tau_y * cos(((double)up + phi_ref) / v.beta));
+    return v.mobility * (fr - tau);
+}
+
+// dt from the CFL rule |v0|max dt / dx = CFL (Sec. 4.3, Sec. 5.2), in FP64
+__device__ __forceinline__ double cfl_dt(double vmax, double cfl, double dx, double dt_max) {
+    double dtd;
+    if (vmax > 0.0) {
+        dtd = cfl * dx / vmax;
+        if (dt_max > 0.0 && dtd > dt_max) dtd = dt_max;
+    } else {
+        dtd = dt_max > 0.0 ? dt_max : 0.0;
+    }
+    return dtd;
+}
+
+// the step's time step: the block's largest |v0| (magnitude bits of a double per thread, NaN
+// above all) into the instance's maximum, and the last of the instance's `ntiles` blocks to
+// finish turns it into dt, once (every block's maximum is in before its fenced increment)
+__device__ __forceinline__ void step_dt_from_max(unsigned long long bits, fdm_dev_scalars* sci, unsigned ntiles,
+                                                 double cfl, double dx, double dt_max) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, bits, o);
+        bits = other > bits ? other : bits;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&sci->vmax_bits, bits);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&sci->ri_count, 1u) == ntiles - 1u) {
+            __threadfence();
+            const double vmax = __longlong_as_double((long long)atomicAdd(&sci->vmax_bits, 0ull));
+            const double dtd = cfl_dt(vmax, cfl, dx, dt_max);
+            sci->dt_next = dtd;
+            sci->dt_h_next = dtd / dx;   // the stencil works in cell units
+            sci->ri_count = 0u;
+        }
+    }
+}
+
+template <typename T>
+struct RowArgs {
+    VelLaw<T> vel;
+    int mode;
+    const void* phi0;          // ROW_TAU: the two state buffers (U13 is needed for friction)
+    const void* phi1;
+    fdm_dev_scalars* sc;       // ROW_TAU: scalars of instance 0
+    int gated;
+    int add_sigma;             // FP64: add sc's sigma_bar13 to the mean (the column pass left it out)
+    T offset;                  // ROW_PLAIN: added to every output value
+    double cfl, dx, dt_max;    // ROW_TAU: time-step rule (FP64)
+};
+
+// the FP64 path's transforms in block fixed point (fdm_fix.cu): launch_row_forward, launch_col
+// and launch_row_inverse of double fields
+cudaError_t fix_preload(int side);
+cudaError_t fix_configure(int n1, int n2);
+void fix_row_forward(const Dev& d, const double* src0, const double* src1, cpx<double>* spec, double* partials,
+                     InstCtl ctl, int count, cudaStream_t s);
+void fix_col(const Dev& d, const cpx<double>* in, cpx<double>* out, const ColArgs<double>& a, int count,
+             cudaStream_t s);
+void fix_row_inverse(const Dev& d, const cpx<double>* spec, double* dst, const RowArgs<double>& a, int count,
+                     cudaStream_t s);
+void fix_tables(void* tw, int n, void* pt, int L, cudaStream_t s);
+
+}  // namespace fdm
