@@ -68,6 +68,11 @@ fdm_status build_group(Dev& d, Arena& A, const fdm_params& p, int count, int gat
         return st;
     if ((st = A.alloc((void**)&d.sc, (size_t)count * sizeof(fdm_dev_scalars)))) return st;
     FDM_CK(cudaMemsetAsync(d.sc, 0, (size_t)count * sizeof(fdm_dev_scalars), s));
+    if (!std::is_same<T, float>::value) {
+        const size_t chunk_bytes = (size_t)count * list_chunks(n) * sizeof(unsigned);
+        if ((st = A.alloc((void**)&d.chunks, chunk_bytes))) return st;
+        FDM_CK(cudaMemsetAsync(d.chunks, 0, chunk_bytes, s));
+    }
     FDM_CK(cudaMemsetAsync(d.phi[0], 0, cn * sizeof(T), s));
     if ((st = upload_twiddles<T>(d.tw1, p.n1, s))) return st;
     if ((st = upload_twiddles<T>(d.tw2, p.n2, s))) return st;
@@ -449,7 +454,8 @@ size_t fdm_device_bytes(const fdm_params* p) {
     size_t n = (size_t)p->n1 * p->n2, e = elt_size(p);
     size_t nk = (size_t)(p->n1 / 2 + 1) * (p->n2 / 2 + 1);
     const size_t lo = p->precision == FDM_MIXED ? 2 * n * sizeof(float) : 0;   // low words of the state
-    return 5 * n * e + lo + nk * e + (size_t)(p->n1 + p->n2) * 4 * e + (size_t)p->n2 * sizeof(double) + 64 * 1024;
+    const size_t list = p->precision == FDM_MIXED ? 0 : list_chunks(n) * sizeof(unsigned);
+    return 5 * n * e + lo + list + nk * e + (size_t)(p->n1 + p->n2) * 4 * e + (size_t)p->n2 * sizeof(double) + 64 * 1024;
 }
 
 fdm_status fdm_create(const fdm_params* p, void* stream, fdm_handle** out) {

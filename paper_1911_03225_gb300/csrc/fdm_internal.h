@@ -21,9 +21,13 @@ struct fdm_dev_scalars {
     unsigned int ri_count;         // blocks of the inverse row kernel that have finished
     long long steps_left;          // gated (batched) launches: steps this instance may still take
     double dt_next, dt_h_next;     // dt of the step being taken and dt / dx (set with max |v0|)
+    unsigned int defer_count;      // nodes on the instance's list in the stencil kernel (see there)
+    unsigned int end_count;        // blocks of the stencil kernel that are done with their tile
 };
 
 constexpr int kKernelsPerStep = 4;
+// chunks of at least 32 entries of a list of n nodes (the stencil's, see knp_step_body)
+inline size_t list_chunks(size_t n) { return n / 32 + 1; }
 constexpr int kKnpShapes = 4;  // stencil block shapes per precision (shape 0 = default)
 
 struct LaunchGeom {
@@ -60,6 +64,7 @@ struct Dev {
     double* red_host;      // pinned host copy: the instance's scalars, then the partials
     int red_blocks;
     fdm_dev_scalars* sc;   // [count]
+    unsigned* chunks;      // [count][list_chunks(n)]: entries in each chunk of the stencil's list
     double phi_ref_host;   // single instance: host copy of sc[0].phi_ref
 };
 

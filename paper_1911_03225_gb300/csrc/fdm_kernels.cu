@@ -382,6 +382,11 @@ struct KnpArgs {
     int time_level;
     fdm_dev_scalars* sc;     // scalars of instance 0
     int gated;
+    int gather;              // collect the warps' left-over nodes in the instances' lists
+    unsigned* list;          // instance 0's list (y n1 + x); the next one list_stride on
+    size_t list_stride;
+    unsigned* chunks;        // entries in each chunk of instance 0's list; the next chunk_stride on
+    size_t chunk_stride;
 };
 
 // Stencil block shapes: block (TX, ty) threads, each updating npt nodes stacked along x2,
@@ -402,7 +407,19 @@ template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed 
 };
 
 // grid (n1 / tx, n2 / (ty npt), instances); block (tx, ty); thread (i, j) updates the
-// nodes (bx + i, by + j + k ty), k < npt
+// nodes (bx + i, by + j + k ty), k < npt.  FP64 and double words: first the nodes that have one
+// characteristic direction (knp_upwind), nearly all of them on the fields the method meets; each
+// warp lists its others and works through them with the whole scheme (knp_node), 32 (or 64) at a
+// time.  What is left over, seldom a full warp's worth, goes on the instance's list in global
+// memory when the launch has several waves of blocks (the list lies in the spectrum's buffer,
+// free between the inverse row kernel and the next step's forward one): the warp that completes
+// a chunk of 32 (64) of the list works through it, and the instance's last block takes the rest.
+// On a launch that the GPU holds at once there are idle lanes to spare, and a tail would cost a
+// scheme's latency (25 us in FP64): each warp sees to its own.  No barrier follows the tile's
+// loads, so warps at the whole scheme and warps at the short one share the pipes.  A node's
+// result depends on the node alone, not on the lists.  2048^2, random field after 30 steps: FP64
+// 1388 -> 624 us, double words 348 -> 245 us (one list per block, behind a barrier: 733 and 369;
+// per warp only: 759 and 426).
 // body of one block: the tile (tbx, tby) of instance inst, ntiles tiles per instance (the
 // last to start advances the clock); thread (tx_, ty_) of a tx x TY block
 template <typename T, int V>
@@ -420,6 +437,9 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
     __shared__ T s_tau[TY * NPT][TX];
     __shared__ T s_dt;
     __shared__ int s_run, s_cur;
+    // per warp: the nodes that need the whole scheme, as row * TX + column
+    __shared__ unsigned short s_list[kPair ? 1 : TY][kPair ? 1 : NPT * TX];
+    __shared__ int s_ended;   // warps done with their part of the tile
     const int rows = TY * npt;
     const int bx = tbx * tx, by = tby * rows;
     const int tid = ty_ * tx + tx_;
@@ -430,6 +450,7 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
         inst_state(ctl, inst, &run, &cur);
         s_run = run;
         s_cur = cur;
+        s_ended = 0;
         if (run) {
             // dt / h of this step, set by the inverse row kernel from max |v0|; the last block
             // of this instance to read it advances the clock, flips the state buffer and clears
@@ -519,36 +540,152 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 lo_out[(size_t)yb * n1 + x] = lo;
             }
         }
-    } else if constexpr (std::is_same<T, df>::value) {
-        // two nodes per pass in the lanes of the packed FP32 instructions (double words), an
-        // odd last node paired with itself and written once
-#pragma unroll 1
-        for (int k = 0; k < npt; k += 2) {
-            const int k2 = (k + 1 < npt) ? k + 1 : k;
-            const int ya = by + ty_ + k * TY, yb = by + ty_ + k2 * TY;
-            const int la = ty_ + k * TY + 2, lb = ty_ + k2 * TY + 2;
-            T va = celerity(a.vel, s_tau[la - 2][tx_], tile[la][lx], phi_ref);
-            T vb = celerity(a.vel, s_tau[lb - 2][tx_], tile[lb][lx], phi_ref);
-            if (a.vel.mfac) {
-                va = va * a.vel.mfac[inst * nn + (size_t)ya * n1 + x];
-                vb = vb * a.vel.mfac[inst * nn + (size_t)yb * n1 + x];
-            }
-            auto f = [&](int i, int j) -> df2 { return mkdf2(tile[la + j][lx + i], tile[lb + j][lx + i]); };
-            const df2 res = knp_node_df2(f, mkdf2(va, vb), dt, a.theta, a.theta_code, a.time_level);
-            out[(size_t)ya * n1 + x] = lane(res, 0);
-            if (k2 != k) out[(size_t)yb * n1 + x] = lane(res, 1);
-        }
     } else {
+        unsigned short* list = s_list[tid >> 5];
+        const unsigned below = (1u << (tid & 31)) - 1u;
+        int count = 0;   // entries on the warp's list
+        auto defer = [&](bool d, int row) {
+            const unsigned m = __ballot_sync(0xffffffffu, d);
+            if (d) list[count + __popc(m & below)] = (unsigned short)(row * TX + tx_);
+            count += __popc(m);
+        };
+        auto place = [&](int row, int col) -> size_t { return (size_t)(by + row) * n1 + bx + col; };
+        // celerity of node o of the field, from its tau13 and U13
+        auto velocity = [&](size_t o, T t, T v) -> T {
+            T c = celerity(a.vel, t, v, phi_ref);
+            if (a.vel.mfac) c = c * a.vel.mfac[inst * nn + o];
+            return c;
+        };
+        constexpr bool kTwo = std::is_same<T, df>::value;   // two nodes at once
+        constexpr int kRound = kTwo ? 64 : 32;              // nodes a warp takes at a time
+        if constexpr (kTwo) {
+            // in the lanes of the packed FP32 instructions (double words), an odd last node paired
+            // with itself and written once
 #pragma unroll 1
-        for (int k = 0; k < npt; ++k) {
-            const int y = by + ty_ + k * TY;
-            const int ly = ty_ + k * TY + 2;
-            const T tau_k = s_tau[ty_ + k * TY][tx_];
-            const T up = tile[ly][lx];
-            T v0 = celerity(a.vel, tau_k, up, phi_ref);
-            if (a.vel.mfac) v0 = v0 * a.vel.mfac[inst * nn + (size_t)y * n1 + x];
-            auto f = [&](int i, int j) -> T { return tile[ly + j][lx + i]; };
-            out[(size_t)y * n1 + x] = knp_node<T>(f, v0, dt, a.theta, a.theta_code, a.time_level);
+            for (int k = 0; k < npt; k += 2) {
+                const int k2 = (k + 1 < npt) ? k + 1 : k;
+                const int ra = ty_ + k * TY, rb = ty_ + k2 * TY, la = ra + 2, lb = rb + 2;
+                auto f = [&](int i, int j) -> df2 { return mkdf2(tile[la + j][lx + i], tile[lb + j][lx + i]); };
+                auto fd = [&](int l, int i, int j) -> df { return tile[(l == 0 ? la : lb) + j][lx + i]; };
+                const size_t oa = place(ra, tx_), ob = place(rb, tx_);
+                const df2 v0 = mkdf2(velocity(oa, s_tau[ra][tx_], tile[la][lx]), velocity(ob, s_tau[rb][tx_], tile[lb][lx]));
+                bool oka, okb;
+                const df2 res = knp_upwind_df2(f, fd, v0, dt, a.theta, a.theta_code, a.time_level, &oka, &okb);
+                if (oka) out[oa] = lane(res, 0);
+                if (okb && k2 != k) out[ob] = lane(res, 1);
+                defer(!oka, ra);
+                defer(!okb && k2 != k, rb);
+            }
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < npt; ++k) {
+                const int r = ty_ + k * TY, ly = r + 2;
+                auto f = [&](int i, int j) -> T { return tile[ly + j][lx + i]; };
+                const size_t o = place(r, tx_);
+                T res;
+                const bool ok = knp_upwind(f, velocity(o, s_tau[r][tx_], tile[ly][lx]), dt, a.theta, a.theta_code,
+                                           a.time_level, &res);
+                if (ok) out[o] = res;
+                defer(!ok, r);
+            }
+        }
+        __syncwarp();
+        const int ln = tid & 31;
+        unsigned* glist = a.list + inst * a.list_stride;
+        unsigned* chunks = a.chunks + inst * a.chunk_stride;
+        // own: the first nodes of the warp's list, in rounds; the rest joins the instance's list
+        const int own = a.gather ? count / kRound * kRound : count, rest = count - own;
+        int done = 0;                  // of the warp's own
+        int todo[2] = {-1, -1};        // chunks of the instance's list this warp completed
+        int tail = 0, tail_chunk = 0;  // the instance's last block: entries of the unfinished chunk
+        if (rest > 0) {
+            unsigned base = 0;
+            if (ln == 0) base = atomicAdd(&sc->defer_count, (unsigned)rest);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            for (int i = ln; i < rest; i += 32) {
+                const int e = list[own + i];
+                glist[base + i] = (unsigned)((by + e / TX) * n1 + bx + e % TX);
+            }
+            __threadfence();   // the entries before their chunk's count
+            __syncwarp();
+            const unsigned c0 = base / kRound, split = min((unsigned)rest, (c0 + 1) * kRound - base);
+            if (ln < 2) {      // at most two chunks touched: lane l sees to chunk c0 + l
+                const unsigned k = ln == 0 ? split : (unsigned)rest - split;
+                if (k > 0 && atomicAdd(&chunks[c0 + ln], k) + k == (unsigned)kRound) {
+                    chunks[c0 + ln] = 0u;
+                    todo[0] = (int)(c0 + ln);
+                }
+            }
+            __threadfence();
+            const int mine = todo[0];
+            todo[0] = __shfl_sync(0xffffffffu, mine, 0);
+            todo[1] = __shfl_sync(0xffffffffu, mine, 1);
+        }
+        // one call site for every source (the scheme's code is large)
+        bool ended = false;
+        while (true) {
+            int m, c = -1;   // nodes of this round; their chunk, or the warp's own list
+            if (done < own) m = min(kRound, own - done);
+            else if (todo[0] >= 0) { c = todo[0]; todo[0] = -1; m = kRound; }
+            else if (todo[1] >= 0) { c = todo[1]; todo[1] = -1; m = kRound; }
+            else if (!ended && a.gather) {
+                ended = true;
+                if (ln == 0) {
+                    __threadfence();
+                    if (atomicAdd(&s_ended, 1) == ((tx * TY) >> 5) - 1) {   // the block's last warp
+                        __threadfence();
+                        if (atomicAdd(&sc->end_count, 1u) == (unsigned)ntiles - 1u) {   // the instance's last block
+                            __threadfence();
+                            const unsigned t = atomicAdd(&sc->defer_count, 0u);
+                            tail_chunk = (int)(t / kRound);
+                            tail = (int)(t % kRound);
+                            chunks[tail_chunk] = 0u;
+                            sc->defer_count = 0u;
+                            sc->end_count = 0u;
+                        }
+                    }
+                }
+                tail = __shfl_sync(0xffffffffu, tail, 0);
+                tail_chunk = __shfl_sync(0xffffffffu, tail_chunk, 0);
+                if (tail == 0) break;
+                c = tail_chunk;
+                m = tail;
+            } else break;
+            auto node = [&](int i, int* x, int* y) {
+                if (c < 0) {
+                    const int e = list[done + i];
+                    *x = bx + e % TX;
+                    *y = by + e / TX;
+                } else {
+                    const unsigned k = __ldcg(glist + (size_t)c * kRound + i);
+                    *x = (int)(k & (unsigned)(n1 - 1));
+                    *y = (int)(k / (unsigned)n1);
+                }
+            };
+            const int mx = n1 - 1, my = n2 - 1;
+            auto at = [&](int x, int y, int i, int j) -> T { return phi[(size_t)((y + j) & my) * n1 + ((x + i) & mx)]; };
+            if constexpr (kTwo) {
+                if (2 * ln < m) {
+                    int xa, ya, xb, yb;
+                    node(2 * ln, &xa, &ya);
+                    node(2 * ln + 1 < m ? 2 * ln + 1 : 2 * ln, &xb, &yb);
+                    const size_t oa = (size_t)ya * n1 + xa, ob = (size_t)yb * n1 + xb;
+                    auto f = [&](int i, int j) -> df2 { return mkdf2(at(xa, ya, i, j), at(xb, yb, i, j)); };
+                    const df2 v0 = mkdf2(velocity(oa, tau[oa], phi[oa]), velocity(ob, tau[ob], phi[ob]));
+                    const df2 res = knp_node_df2(f, v0, dt, a.theta, a.theta_code, a.time_level);
+                    out[oa] = lane(res, 0);
+                    if (ob != oa) out[ob] = lane(res, 1);
+                }
+            } else {
+                if (ln < m) {
+                    int x, y;
+                    node(ln, &x, &y);
+                    const size_t o = (size_t)y * n1 + x;
+                    auto f = [&](int i, int j) -> T { return at(x, y, i, j); };
+                    out[o] = knp_node<T>(f, velocity(o, tau[o], phi[o]), dt, a.theta, a.theta_code, a.time_level);
+                }
+            }
+            if (c < 0) done += m;
         }
     }
 }
@@ -981,12 +1118,14 @@ void launch_row_inverse(const Dev& d, const cpx<T>* spec, T* dst, int mode, doub
 }
 
 template <typename T, int V>
-void launch_knp_shape(const Dev& d, const KnpArgs<T>& a, cudaStream_t s) {
+void launch_knp_shape(const Dev& d, KnpArgs<T> a, cudaStream_t s) {
     constexpr int TY = KnpShapes<T>::ty[V];
     const int tx = d.p.n1 < TX ? d.p.n1 : TX;
     int npt = KnpShapes<T>::npt[V];
     while (npt > 1 && d.p.n2 < TY * npt) npt >>= 1;
     dim3 grid(d.p.n1 / tx, d.p.n2 / (TY * npt), d.count), block(tx, TY);
+    // two blocks of 256 threads to an SM: several waves from here on
+    a.gather = (size_t)grid.x * grid.y * grid.z * tx * TY > (size_t)2 * 152 * 2 * 256 ? 1 : 0;
     knp_step_kernel<T, V><<<grid, block, 0, s>>>((const T*)d.phi[0], (const T*)d.phi[1], (const T*)d.tau,
                                                  d.p.n1, d.p.n2, npt, a);
 }
@@ -1002,6 +1141,12 @@ KnpArgs<T> knp_args(const Dev& d) {
     a.time_level = d.p.time_level;
     a.sc = d.sc;
     a.gated = d.gated;
+    const size_t n = (size_t)d.p.n1 * d.p.n2;
+    a.gather = 0;   // set with the grid
+    a.list = static_cast<unsigned*>(d.spec);
+    a.list_stride = n * sizeof(T) / sizeof(unsigned);
+    a.chunks = d.chunks;
+    a.chunk_stride = list_chunks(n);
     return a;
 }
 template <typename T>
