@@ -120,18 +120,18 @@ fdm_status fdm_batch_set_plastic_distortion(fdm_batch* b, int32_t i, const doubl
     if (!index_ok(b, i) || !up13) return FDM_ERR_INVALID_ARG;
     auto& G = b->groups[b->group_of[i]];
     const int j = b->local_of[i];
-    const size_t n = (size_t)G.d.p.n1 * G.d.p.n2;
-    double mean = ksum(up13, n) / (double)n;
-    if (!std::isfinite(mean)) return FDM_ERR_INVALID_ARG;
+    fdm_dev_scalars now;
+    FDM_CK(cudaMemcpyAsync(&now, G.d.sc + j, sizeof(now), cudaMemcpyDeviceToHost, b->stream));
     FDM_CK(cudaStreamSynchronize(b->stream));
+    double mean = 0.0;
+    int cur = now.cur;
+    if (fdm_status st = set_state(G.d, G.prec, j, up13, &cur, &mean, b->stream)) return st;
     const double ref = G.prec != FDM_FP64 ? mean : 0.0;
-    fdm_status st = upload_state(G.d, G.prec, 0, j, up13, ref, b->stream);
-    if (st) return st;
     fdm_dev_scalars s;
     std::memset(&s, 0, sizeof(s));
     s.phi_ref = ref;
     s.mean_up13 = mean;
-    s.cur = 0;
+    s.cur = cur;
     s.steps_left = 0;
     host_loading(G.d.p, 0, 0.0, mean, &s.eps_bar13, &s.sigma_bar13);
     FDM_CK(cudaMemcpyAsync(G.d.sc + j, &s, sizeof(s), cudaMemcpyHostToDevice, b->stream));
@@ -275,7 +275,8 @@ fdm_status fdm_batch_read_fields(fdm_batch* b, int32_t i, uint32_t mask, double*
     if (mask & FDM_FIELD_UP13)
         if ((st = download_state(up13, G.d, G.prec, s.cur, j, G.phi_ref[j], b->stream))) return st;
     if (mask & FDM_FIELD_TAU13)
-        if ((st = download_field(tau13, (char*)G.d.tau + (size_t)j * n * e, n, G.prec, 0.0, b->stream)))
+        if ((st = download_field(tau13, (char*)G.d.tau + (size_t)j * n * e, n, G.prec, 0.0,
+                                 state_stage(G.d, G.prec, j, 1 - s.cur), b->stream)))
             return st;
     return FDM_OK;
 }

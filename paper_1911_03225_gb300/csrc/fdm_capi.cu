@@ -108,80 +108,160 @@ template fdm_status build_group<double>(Dev&, Arena&, const fdm_params&, int, in
 template fdm_status build_group<float>(Dev&, Arena&, const fdm_params&, int, int, bool, cudaStream_t);
 template fdm_status build_group<df>(Dev&, Arena&, const fdm_params&, int, int, bool, cudaStream_t);
 
-fdm_status upload_field(void* dst, const double* src, size_t n, int prec, double offset, cudaStream_t s) {
+Stage state_stage(const Dev& d, int prec, int inst, int b) {
+    const size_t n = (size_t)d.p.n1 * d.p.n2;
+    if (prec != FDM_MIXED) return Stage{{(double*)((char*)d.phi[b] + inst * n * 8), nullptr}, {n, 0}};
+    return Stage{{(double*)((float*)d.phi[b] + inst * n), (double*)((float*)d.phi_lo[b] + inst * n)}, {n / 2, n / 2}};
+}
+
+// the spectra of a single instance as a stage (dead but for the steps' phases 0 to 2)
+static Stage spectrum_stage(const Dev& d, int prec) {
+    const size_t n = (size_t)d.p.n1 * d.p.n2;
+    if (prec != FDM_MIXED) return Stage{{(double*)d.spec, nullptr}, {n, 0}};
+    return Stage{{(double*)d.spec, (double*)d.spec2}, {n / 2, n / 2}};
+}
+
+fdm_status stage_upload(const Stage& g, const double* src, double* red, double* red_host, int nblk, FieldStats* st,
+                        cudaStream_t s) {
+    st->sum = st->top = 0.0;
+    st->low = HUGE_VAL;
+    std::vector<double> parts;
+    for (int k = 0; k < 2; ++k) {
+        if (g.len[k] == 0) continue;
+        FDM_CK(cudaMemcpyAsync(g.piece[k], src + (k ? g.len[0] : 0), g.len[k] * sizeof(double), cudaMemcpyHostToDevice, s));
+        launch_field_stats(g.piece[k], g.len[k], red, nblk, s);
+        FDM_CK(cudaGetLastError());
+        FDM_CK(cudaMemcpyAsync(red_host, red, (size_t)4 * nblk * sizeof(double), cudaMemcpyDeviceToHost, s));
+        FDM_CK(cudaStreamSynchronize(s));
+        for (int q = 0; q < nblk; ++q) {
+            parts.push_back(red_host[4 * q]);
+            parts.push_back(red_host[4 * q + 1]);
+            const double top = red_host[4 * q + 2], low = red_host[4 * q + 3];
+            if (!std::isnan(st->top) && !(top <= st->top)) st->top = top;   // a NaN stays
+            if (low < st->low) st->low = low;
+        }
+    }
+    st->sum = ksum(parts.data(), parts.size());
+    return FDM_OK;
+}
+
+fdm_status stage_convert(const Stage& g, void* dst, int prec, double offset, cudaStream_t s) {
+    for (int k = 0; k < 2; ++k) {
+        if (g.len[k] == 0) continue;
+        const size_t at = k ? g.len[0] : 0;
+        FDM_DISPATCH(prec, launch_convert<T>(g.piece[k], (T*)dst + at, g.len[k], offset, s));
+    }
+    FDM_CK(cudaGetLastError());
+    return FDM_OK;
+}
+
+fdm_status upload_field(void* dst, const double* src, size_t n, int prec, double offset, const Stage& stage,
+                        cudaStream_t s) {
     if (prec == FDM_FP64 && offset == 0.0) {
         FDM_CK(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyHostToDevice, s));
         FDM_CK(cudaStreamSynchronize(s));
         return FDM_OK;
     }
-    if (prec == FDM_MIXED) {
-        std::vector<float> t(n);
-        for (size_t i = 0; i < n; ++i) t[i] = (float)(src[i] - offset);
-        FDM_CK(cudaMemcpyAsync(dst, t.data(), n * sizeof(float), cudaMemcpyHostToDevice, s));
-        FDM_CK(cudaStreamSynchronize(s));
-        return FDM_OK;
+    for (int k = 0; k < 2; ++k) {
+        if (stage.len[k] == 0) continue;
+        FDM_CK(cudaMemcpyAsync(stage.piece[k], src + (k ? stage.len[0] : 0), stage.len[k] * sizeof(double),
+                               cudaMemcpyHostToDevice, s));
     }
-    if (prec == FDM_DF64) {
-        std::vector<df> t(n);
-        for (size_t i = 0; i < n; ++i) t[i] = df(src[i] - offset);
-        FDM_CK(cudaMemcpyAsync(dst, t.data(), n * sizeof(df), cudaMemcpyHostToDevice, s));
-        FDM_CK(cudaStreamSynchronize(s));
-        return FDM_OK;
-    }
-    std::vector<double> t(n);
-    for (size_t i = 0; i < n; ++i) t[i] = src[i] - offset;
-    FDM_CK(cudaMemcpyAsync(dst, t.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
+    fdm_status st = stage_convert(stage, dst, prec, offset, s);
+    if (st) return st;
     FDM_CK(cudaStreamSynchronize(s));
     return FDM_OK;
 }
 
-fdm_status download_field(double* dst, const void* src, size_t n, int prec, double offset, cudaStream_t s) {
-    if (prec == FDM_MIXED) {
-        std::vector<float> t(n);
-        FDM_CK(cudaMemcpyAsync(t.data(), src, n * sizeof(float), cudaMemcpyDeviceToHost, s));
+fdm_status download_field(double* dst, const void* src, size_t n, int prec, double offset, const Stage& stage,
+                          cudaStream_t s) {
+    if (prec == FDM_FP64) {
+        FDM_CK(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyDeviceToHost, s));
         FDM_CK(cudaStreamSynchronize(s));
-        for (size_t i = 0; i < n; ++i) dst[i] = (double)t[i] + offset;
+        if (offset != 0.0)
+            for (size_t i = 0; i < n; ++i) dst[i] += offset;
         return FDM_OK;
     }
-    if (prec == FDM_DF64) {
-        std::vector<df> t(n);
-        FDM_CK(cudaMemcpyAsync(t.data(), src, n * sizeof(df), cudaMemcpyDeviceToHost, s));
-        FDM_CK(cudaStreamSynchronize(s));
-        for (size_t i = 0; i < n; ++i) dst[i] = (double)t[i] + offset;
-        return FDM_OK;
+    for (int k = 0; k < 2; ++k) {
+        if (stage.len[k] == 0) continue;
+        const size_t at = k ? stage.len[0] : 0;
+        FDM_DISPATCH(prec, launch_merge<T>((const T*)src + at, nullptr, stage.piece[k], stage.len[k], offset, s));
+        FDM_CK(cudaGetLastError());
+        FDM_CK(cudaMemcpyAsync(dst + at, stage.piece[k], stage.len[k] * sizeof(double), cudaMemcpyDeviceToHost, s));
     }
-    FDM_CK(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyDeviceToHost, s));
     FDM_CK(cudaStreamSynchronize(s));
-    if (offset != 0.0)
-        for (size_t i = 0; i < n; ++i) dst[i] += offset;
     return FDM_OK;
 }
 
-fdm_status upload_state(const Dev& d, int prec, int b, int inst, const double* src, double offset, cudaStream_t s) {
+// small fields: converted on the host, into buffer 0
+static fdm_status set_state_host(const Dev& d, int prec, int inst, const double* src, int* cur, double* mean,
+                                 cudaStream_t s) {
     const size_t n = (size_t)d.p.n1 * d.p.n2;
-    if (prec != FDM_MIXED)
-        return upload_field((char*)d.phi[b] + (size_t)inst * n * elt_size(&d.p), src, n, prec, offset, s);
-    std::vector<float> hi(n), lo(n);
-    for (size_t i = 0; i < n; ++i) {
-        const double v = src[i] - offset;
-        hi[i] = (float)v;
-        lo[i] = (float)(v - (double)hi[i]);
+    *mean = ksum(src, n) / (double)n;
+    if (!std::isfinite(*mean)) return FDM_ERR_INVALID_ARG;
+    if (prec == FDM_FP64) {
+        FDM_CK(cudaMemcpyAsync((double*)d.phi[0] + inst * n, src, n * sizeof(double), cudaMemcpyHostToDevice, s));
+    } else if (prec == FDM_DF64) {
+        std::vector<df> t(n);
+        for (size_t i = 0; i < n; ++i) t[i] = df(src[i] - *mean);
+        FDM_CK(cudaMemcpyAsync((df*)d.phi[0] + inst * n, t.data(), n * sizeof(df), cudaMemcpyHostToDevice, s));
+        FDM_CK(cudaStreamSynchronize(s));
+    } else {
+        std::vector<float> hi(n), lo(n);
+        for (size_t i = 0; i < n; ++i) {
+            const double v = src[i] - *mean;
+            hi[i] = (float)v;
+            lo[i] = (float)(v - (double)hi[i]);
+        }
+        FDM_CK(cudaMemcpyAsync((float*)d.phi[0] + inst * n, hi.data(), n * sizeof(float), cudaMemcpyHostToDevice, s));
+        FDM_CK(cudaMemcpyAsync((float*)d.phi_lo[0] + inst * n, lo.data(), n * sizeof(float), cudaMemcpyHostToDevice, s));
+        FDM_CK(cudaStreamSynchronize(s));
     }
-    FDM_CK(cudaMemcpyAsync((float*)d.phi[b] + inst * n, hi.data(), n * sizeof(float), cudaMemcpyHostToDevice, s));
-    FDM_CK(cudaMemcpyAsync((float*)d.phi_lo[b] + inst * n, lo.data(), n * sizeof(float), cudaMemcpyHostToDevice, s));
     FDM_CK(cudaStreamSynchronize(s));
+    *cur = 0;
+    return FDM_OK;
+}
+
+fdm_status set_state(const Dev& d, int prec, int inst, const double* src, int* cur, double* mean, cudaStream_t s) {
+    const size_t n = (size_t)d.p.n1 * d.p.n2;
+    if (n < kHostField) return set_state_host(d, prec, inst, src, cur, mean, s);
+    // the doubles arrive in the buffer that is not the state, so a refused field leaves it alone
+    const Stage g = state_stage(d, prec, inst, 1 - *cur);
+    double* red_host = (double*)((char*)d.red_host + kInfoScalarBytes);
+    FieldStats fs;
+    fdm_status st = stage_upload(g, src, d.red, red_host, d.red_blocks, &fs, s);
+    if (st) return st;
+    *mean = fs.sum / (double)n;
+    if (!std::isfinite(*mean) || !std::isfinite(fs.top)) return FDM_ERR_INVALID_ARG;
+    if (prec == FDM_FP64) {   // they are the new state
+        *cur = 1 - *cur;
+        return FDM_OK;
+    }
+    if (prec == FDM_DF64) {
+        launch_convert<df>(g.piece[0], (df*)d.phi[*cur] + inst * n, n, *mean, s);
+    } else {
+        for (int k = 0; k < 2; ++k) {
+            const size_t at = inst * n + (k ? g.len[0] : 0);
+            launch_split_pair(g.piece[k], (float*)d.phi[*cur] + at, (float*)d.phi_lo[*cur] + at, g.len[k], *mean, s);
+        }
+    }
+    FDM_CK(cudaGetLastError());
     return FDM_OK;
 }
 
 fdm_status download_state(double* dst, const Dev& d, int prec, int b, int inst, double offset, cudaStream_t s) {
     const size_t n = (size_t)d.p.n1 * d.p.n2;
+    const Stage g = state_stage(d, prec, inst, 1 - b);
     if (prec != FDM_MIXED)
-        return download_field(dst, (const char*)d.phi[b] + (size_t)inst * n * elt_size(&d.p), n, prec, offset, s);
-    std::vector<float> hi(n), lo(n);
-    FDM_CK(cudaMemcpyAsync(hi.data(), (const float*)d.phi[b] + inst * n, n * sizeof(float), cudaMemcpyDeviceToHost, s));
-    FDM_CK(cudaMemcpyAsync(lo.data(), (const float*)d.phi_lo[b] + inst * n, n * sizeof(float), cudaMemcpyDeviceToHost, s));
+        return download_field(dst, (const char*)d.phi[b] + (size_t)inst * n * elt_size(&d.p), n, prec, offset, g, s);
+    for (int k = 0; k < 2; ++k) {
+        const size_t at = k ? g.len[0] : 0;
+        launch_merge<float>((const float*)d.phi[b] + inst * n + at, (const float*)d.phi_lo[b] + inst * n + at,
+                            g.piece[k], g.len[k], offset, s);
+        FDM_CK(cudaGetLastError());
+        FDM_CK(cudaMemcpyAsync(dst + at, g.piece[k], g.len[k] * sizeof(double), cudaMemcpyDeviceToHost, s));
+    }
     FDM_CK(cudaStreamSynchronize(s));
-    for (size_t i = 0; i < n; ++i) dst[i] = ((double)hi[i] + (double)lo[i]) + offset;
     return FDM_OK;
 }
 
@@ -316,12 +396,12 @@ struct fdm_handle {
 
 namespace {
 
-fdm_status reset_scalars(fdm_handle* h, double mean) {
+fdm_status reset_scalars(fdm_handle* h, double mean, int cur) {
     fdm_dev_scalars s;
     std::memset(&s, 0, sizeof(s));
     s.phi_ref = h->d.phi_ref_host;
     s.mean_up13 = mean;
-    s.cur = 0;
+    s.cur = cur;
     s.steps_left = -1;
     host_loading(h->d.p, 0, 0.0, mean, &s.eps_bar13, &s.sigma_bar13);
     FDM_CK(cudaMemcpyAsync(h->d.sc, &s, sizeof(s), cudaMemcpyHostToDevice, h->stream));
@@ -386,10 +466,11 @@ fdm_status read_fields_impl(fdm_handle* h, uint32_t mask, double* up13, double* 
     if ((st = read_scalars(h, &sc))) return st;
     const T* phi = (const T*)d.phi[sc.cur];
     const int mx = h->prec;
+    const Stage stage = state_stage(d, mx, 0, 1 - sc.cur);
     if (mask & FDM_FIELD_UP13)
         if ((st = download_state(up13, d, mx, sc.cur, 0, d.phi_ref_host, h->stream))) return st;
     if (mask & FDM_FIELD_TAU13)
-        if ((st = download_field(tau, d.tau, h->n, mx, 0.0, h->stream))) return st;
+        if ((st = download_field(tau, d.tau, h->n, mx, 0.0, stage, h->stream))) return st;
     const bool nye64 = mx == FDM_MIXED && (mask & (FDM_FIELD_ALPHA11 | FDM_FIELD_ALPHA12));
     if (nye64) {
         if ((st = ensure_readout64(h))) return st;
@@ -398,26 +479,26 @@ fdm_status read_fields_impl(fdm_handle* h, uint32_t mask, double* up13, double* 
         launch_alpha<double>(h->rd64, u64, (double*)h->rd64_buf[1], (double*)h->rd64_buf[2], h->stream);
         FDM_CK(cudaGetLastError());
         if (mask & FDM_FIELD_ALPHA11)
-            if ((st = download_field(a11, h->rd64_buf[1], h->n, FDM_FP64, 0.0, h->stream))) return st;
+            if ((st = download_field(a11, h->rd64_buf[1], h->n, FDM_FP64, 0.0, stage, h->stream))) return st;
         if (mask & FDM_FIELD_ALPHA12)
-            if ((st = download_field(a12, h->rd64_buf[2], h->n, FDM_FP64, 0.0, h->stream))) return st;
+            if ((st = download_field(a12, h->rd64_buf[2], h->n, FDM_FP64, 0.0, stage, h->stream))) return st;
     }
     if ((mask & (FDM_FIELD_V1 | FDM_FIELD_V2)) || (!nye64 && (mask & (FDM_FIELD_ALPHA11 | FDM_FIELD_ALPHA12)))) {
         if ((st = ensure_readout<T>(h))) return st;
         launch_alpha<T>(d, phi, (T*)h->rd[0], (T*)h->rd[1], h->stream);
         FDM_CK(cudaGetLastError());
         if ((mask & FDM_FIELD_ALPHA11) && !nye64)
-            if ((st = download_field(a11, h->rd[0], h->n, mx, 0.0, h->stream))) return st;
+            if ((st = download_field(a11, h->rd[0], h->n, mx, 0.0, stage, h->stream))) return st;
         if ((mask & FDM_FIELD_ALPHA12) && !nye64)
-            if ((st = download_field(a12, h->rd[1], h->n, mx, 0.0, h->stream))) return st;
+            if ((st = download_field(a12, h->rd[1], h->n, mx, 0.0, stage, h->stream))) return st;
         if (mask & (FDM_FIELD_V1 | FDM_FIELD_V2)) {
             launch_velocity<T>(d, (const T*)h->rd[0], (const T*)h->rd[1], (const T*)d.tau, phi, (T*)h->rd[2],
                                (T*)h->rd[3], h->stream);
             FDM_CK(cudaGetLastError());
             if (mask & FDM_FIELD_V1)
-                if ((st = download_field(v1, h->rd[2], h->n, mx, 0.0, h->stream))) return st;
+                if ((st = download_field(v1, h->rd[2], h->n, mx, 0.0, stage, h->stream))) return st;
             if (mask & FDM_FIELD_V2)
-                if ((st = download_field(v2, h->rd[3], h->n, mx, 0.0, h->stream))) return st;
+                if ((st = download_field(v2, h->rd[3], h->n, mx, 0.0, stage, h->stream))) return st;
         }
     }
     return FDM_OK;
@@ -482,63 +563,59 @@ fdm_status fdm_create(const fdm_params* p, void* stream, fdm_handle** out) {
     return FDM_OK;
 }
 
-// FP64 state: the field goes to the device as it is (staged in the stress buffer, which the
-// next static solve overwrites) and its mean comes from a device reduction, so that a large
-// restart costs one copy rather than a host pass; the state is replaced only if the sum is
-// finite.
-static fdm_status set_state_fp64(fdm_handle* h, const double* up13) {
-    Dev& d = h->d;
-    const size_t n = h->n;
-    FDM_CK(cudaStreamSynchronize(h->stream));
-    FDM_CK(cudaMemcpyAsync(d.tau, up13, n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    Dev r = d;
-    r.phi[0] = r.phi[1] = d.tau;
-    r.phi_lo[0] = r.phi_lo[1] = nullptr;
-    r.sc = nullptr;
-    launch_alpha_sums<double>(r, 0, d.red, d.red_blocks, h->stream);
-    FDM_CK(cudaGetLastError());
-    double* part = (double*)((char*)d.red_host + kInfoScalarBytes);
-    FDM_CK(cudaMemcpyAsync(part, d.red, (size_t)6 * d.red_blocks * sizeof(double), cudaMemcpyDeviceToHost,
-                           h->stream));
-    FDM_CK(cudaStreamSynchronize(h->stream));
-    std::vector<double> col(d.red_blocks);
-    for (int b = 0; b < d.red_blocks; ++b) col[b] = part[6 * b + 5];
-    const double mean = ksum(col.data(), col.size()) / (double)n;
-    if (!std::isfinite(mean)) return FDM_ERR_INVALID_ARG;
-    FDM_CK(cudaMemcpyAsync(d.phi[0], d.tau, n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
-    d.phi_ref_host = 0.0;
-    return reset_scalars(h, mean);
-}
-
 fdm_status fdm_set_plastic_distortion(fdm_handle* h, const double* up13) {
     if (!h || !up13) return FDM_ERR_INVALID_ARG;
-    if (h->prec == FDM_FP64) return set_state_fp64(h, up13);
-    double mean = ksum(up13, h->n) / (double)h->n;
-    if (!std::isfinite(mean)) return FDM_ERR_INVALID_ARG;
-    FDM_CK(cudaStreamSynchronize(h->stream));
+    fdm_dev_scalars sc;
+    fdm_status st = read_scalars(h, &sc);
+    if (st) return st;
+    double mean = 0.0;
+    int cur = sc.cur;
+    if ((st = set_state(h->d, h->prec, 0, up13, &cur, &mean, h->stream))) return st;
     // FP32 and double-word storage hold U13 minus its mean (the scheme is offset equivariant)
     h->d.phi_ref_host = h->prec != FDM_FP64 ? mean : 0.0;
-    fdm_status st = upload_state(h->d, h->prec, 0, 0, up13, h->d.phi_ref_host, h->stream);
-    if (st) return st;
-    return reset_scalars(h, mean);
+    return reset_scalars(h, mean, cur);
 }
 
 fdm_status fdm_set_density(fdm_handle* h, const double* a11, const double* a12, double mean_up13,
                            double* div_residual) {
     if (!h || !a11 || !a12 || !std::isfinite(mean_up13)) return FDM_ERR_INVALID_ARG;
     const size_t n = h->n;
-    double m11 = ksum(a11, n) / (double)n, m12 = ksum(a12, n) / (double)n, amax = 0.0;
-    for (size_t i = 0; i < n; ++i) {
-        if (!std::isfinite(a11[i]) || !std::isfinite(a12[i])) return FDM_ERR_INVALID_ARG;
-        amax = std::fmax(amax, std::fmax(std::fabs(a11[i]), std::fabs(a12[i])));
+    Dev& d = h->d;
+    fdm_status st;
+    const Stage spec = spectrum_stage(d, h->prec);
+    // large fields are checked on the device (in the spectra, unless a step's phases still need
+    // them), small ones here
+    const bool on_device = n >= kHostField && h->next_phase == 0;
+    double m11, m12, amax = 0.0;
+    if (on_device) {
+        double* red_host = (double*)((char*)d.red_host + kInfoScalarBytes);
+        FieldStats f1, f2;
+        if ((st = stage_upload(spec, a11, d.red, red_host, d.red_blocks, &f1, h->stream))) return st;
+        // FP64: the second spectrum takes alpha12, so both are on the device already
+        const Stage other = h->prec == FDM_FP64 ? Stage{{(double*)d.spec2, nullptr}, {n, 0}} : spec;
+        if ((st = stage_upload(other, a12, d.red, red_host, d.red_blocks, &f2, h->stream))) return st;
+        if (!std::isfinite(f1.top) || !std::isfinite(f2.top)) return FDM_ERR_INVALID_ARG;
+        m11 = f1.sum / (double)n;
+        m12 = f2.sum / (double)n;
+        amax = std::fmax(f1.top, f2.top);
+    } else {
+        m11 = ksum(a11, n) / (double)n;
+        m12 = ksum(a12, n) / (double)n;
+        for (size_t i = 0; i < n; ++i) {
+            if (!std::isfinite(a11[i]) || !std::isfinite(a12[i])) return FDM_ERR_INVALID_ARG;
+            amax = std::fmax(amax, std::fmax(std::fabs(a11[i]), std::fabs(a12[i])));
+        }
     }
     if (std::fabs(m11) > 1e-9 * amax || std::fabs(m12) > 1e-9 * amax) return FDM_ERR_NET_BURGERS;
     FDM_CK(cudaStreamSynchronize(h->stream));
-    Dev& d = h->d;
-    fdm_status st;
     // stage alpha in the two state buffers (the old state is being replaced)
-    if ((st = upload_field(d.phi[0], a11, n, h->prec, 0.0, h->stream))) return st;
-    if ((st = upload_field(d.phi[1], a12, n, h->prec, 0.0, h->stream))) return st;
+    if (on_device && h->prec == FDM_FP64) {
+        FDM_CK(cudaMemcpyAsync(d.phi[0], d.spec, n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+        FDM_CK(cudaMemcpyAsync(d.phi[1], d.spec2, n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
+    } else {
+        if ((st = upload_field(d.phi[0], a11, n, h->prec, 0.0, spec, h->stream))) return st;
+        if ((st = upload_field(d.phi[1], a12, n, h->prec, 0.0, spec, h->stream))) return st;
+    }
     double phi_ref = h->prec != FDM_FP64 ? mean_up13 : 0.0;
     const int nblk = d.red_blocks;
     FDM_DISPATCH(h->prec, launch_curl_inverse<T>(d, (const T*)d.phi[0], (const T*)d.phi[1], (T*)d.phi[0], mean_up13,
@@ -553,7 +630,7 @@ fdm_status fdm_set_density(fdm_handle* h, const double* a11, const double* a12, 
     if (div_residual) *div_residual = res;
     d.phi_ref_host = phi_ref;
     if (d.phi_lo[0]) FDM_CK(cudaMemsetAsync(d.phi_lo[0], 0, n * sizeof(float), h->stream));
-    if ((st = reset_scalars(h, mean_up13))) return st;
+    if ((st = reset_scalars(h, mean_up13, 0))) return st;
     return res > 1e-6 ? FDM_WARN_NOT_DIV_FREE : FDM_OK;
 }
 
@@ -580,6 +657,35 @@ static fdm_status alloc_hetero(fdm_handle* h) {
     fdm_status st;
     for (int i = 0; i < 6; ++i)
         if (!*bufs[i] && (st = h->arena.alloc(bufs[i], sizes[i]))) return st;
+    return FDM_OK;
+}
+
+static bool valid_modulus(const double* factor, size_t n) {
+    for (size_t i = 0; i < n; ++i)
+        if (!(factor[i] > 0.0) || !std::isfinite(factor[i])) return false;
+    return true;
+}
+// the shear modulus mu * factor of a host field into the handle's buffer, with its mean of the
+// extremes; every factor finite and > 0, else FDM_ERR_INVALID_ARG and the old field kept.  The
+// iterate's buffers, free between solves, take the doubles.
+static fdm_status set_modulus(fdm_handle* h, const double* factor, double* mu0) {
+    const fdm_params& p = h->d.p;
+    const size_t n = h->n;
+    const double mu = p.E / (2.0 * (1.0 + p.nu));
+    const Stage g = h->prec == FDM_MIXED ? Stage{{(double*)h->hetero.g1, (double*)h->hetero.g2}, {n / 2, n / 2}}
+                                         : Stage{{(double*)h->hetero.g1, nullptr}, {n, 0}};
+    FieldStats fs;
+    fdm_status st = stage_upload(g, factor, h->d.red, (double*)((char*)h->d.red_host + kInfoScalarBytes),
+                                 h->d.red_blocks, &fs, h->stream);
+    if (st) return st;
+    if (!std::isfinite(fs.top) || !(fs.low > 0.0)) return FDM_ERR_INVALID_ARG;
+    for (int k = 0; k < 2; ++k) {
+        if (g.len[k] == 0) continue;
+        const size_t at = k ? g.len[0] : 0;
+        FDM_DISPATCH(h->prec, launch_scale<T>(g.piece[k], (T*)h->hetero.mu + at, g.len[k], mu, h->stream));
+    }
+    FDM_CK(cudaGetLastError());
+    *mu0 = 0.5 * (mu * fs.low + mu * fs.top);   // products of positive values are monotone
     return FDM_OK;
 }
 
@@ -617,22 +723,12 @@ fdm_status fdm_set_shear_modulus_field(fdm_handle* h, const double* mu_factor, d
     }
     const fdm_params& p = h->d.p;
     if (p.nh != p.nz || !(tol >= 0.0) || !std::isfinite(tol) || max_iter < 1) return FDM_ERR_INVALID_ARG;
-    const size_t n = h->n;
-    const double mu = p.E / (2.0 * (1.0 + p.nu));
-    std::vector<double> m(n);
-    double mmin = HUGE_VAL, mmax = 0.0;
-    for (size_t i = 0; i < n; ++i) {
-        if (!(mu_factor[i] > 0.0) || !std::isfinite(mu_factor[i])) return FDM_ERR_INVALID_ARG;
-        m[i] = mu * mu_factor[i];
-        mmin = std::fmin(mmin, m[i]);
-        mmax = std::fmax(mmax, m[i]);
-    }
-    if (h->next_phase != 0) return FDM_ERR_STATE;
+    if (h->next_phase != 0) return valid_modulus(mu_factor, h->n) ? FDM_ERR_STATE : FDM_ERR_INVALID_ARG;
     fdm_status st;
     if ((st = alloc_hetero(h))) return st;
     FDM_CK(cudaStreamSynchronize(h->stream));
-    if ((st = upload_field(h->hetero.mu, m.data(), n, h->prec, 0.0, h->stream))) return st;
-    h->hetero_mu0 = 0.5 * (mmin + mmax);
+    if ((st = set_modulus(h, mu_factor, &h->hetero_mu0))) return st;
+    FDM_CK(cudaStreamSynchronize(h->stream));
     h->hetero_tol = tol;
     h->hetero_max_iter = max_iter;
     h->hetero_on = true;
@@ -753,7 +849,9 @@ static fdm_status read_stress_planes(fdm_handle* h, int32_t comp, int32_t nplane
     // into i sin; the unpaired x3 Nyquist term is dropped
     const bool odd3 = comp != FDM_S13 && comp != FDM_S23;
     std::vector<double> w((size_t)p.nz / 2 + 1);
-    std::vector<double> host((size_t)h->n);
+    fdm_dev_scalars now;
+    if ((st = read_scalars(h, &now))) return st;
+    const Stage stage = state_stage(h->d, h->prec, 0, 1 - now.cur);
     for (int32_t k = 0; k < nplanes; ++k) {
         // weights D(k3) cos (or sin) of 2 pi k3 (x3 - (nh - 1)/2) / nz, k3 in [0, nz/2]
         const double shift = (double)planes[k] - 0.5 * (double)(p.nh - 1);
@@ -785,8 +883,8 @@ static fdm_status read_stress_planes(fdm_handle* h, int32_t comp, int32_t nplane
                          launch_stress_to<T>(r, comp, (T*)h->plane_buf[3], h->stream));
         }
         FDM_CK(cudaGetLastError());
-        if ((st = download_field(host.data(), h->plane_buf[3], h->n, h->prec, 0.0, h->stream))) return st;
-        std::memcpy(out + (size_t)k * h->n, host.data(), h->n * sizeof(double));
+        if ((st = download_field(out + (size_t)k * h->n, h->plane_buf[3], h->n, h->prec, 0.0, stage, h->stream)))
+            return st;
     }
     return FDM_OK;
 }
@@ -797,19 +895,11 @@ fdm_status fdm_static_solve_heterogeneous(fdm_handle* h, const double* mu_factor
     const fdm_params& p = h->d.p;
     if (p.nh != p.nz) return FDM_ERR_INVALID_ARG;
     const size_t n = h->n;
-    const double mu = p.E / (2.0 * (1.0 + p.nu));
-    std::vector<double> m(n);
-    double mmin = HUGE_VAL, mmax = 0.0;
-    for (size_t i = 0; i < n; ++i) {
-        if (!(mu_factor[i] > 0.0) || !std::isfinite(mu_factor[i])) return FDM_ERR_INVALID_ARG;
-        m[i] = mu * mu_factor[i];
-        mmin = std::fmin(mmin, m[i]);
-        mmax = std::fmax(mmax, m[i]);
-    }
-    if (!h->has_state || h->next_phase != 0) return FDM_ERR_STATE;
+    if (!h->has_state || h->next_phase != 0) return valid_modulus(mu_factor, n) ? FDM_ERR_STATE : FDM_ERR_INVALID_ARG;
     fdm_status st;
     if ((st = alloc_hetero(h))) return st;
-    if ((st = upload_field(h->hetero.mu, m.data(), n, h->prec, 0.0, h->stream))) return st;
+    double mu0 = 0.0;
+    if ((st = set_modulus(h, mu_factor, &mu0))) return st;
     // the loading of the current step: sigma_bar13 (stress, zero mean stress) or eps_bar13
     fdm_dev_scalars s;
     if ((st = read_scalars(h, &s))) return st;
@@ -818,16 +908,17 @@ fdm_status fdm_static_solve_heterogeneous(fdm_handle* h, const double* mu_factor
     const bool stress = p.loading_mode == FDM_LOAD_STRESS || p.loading_mode == FDM_LOAD_ZERO_MEAN_STRESS;
     int it = 0;
     double r = 0.0;
-    FDM_DISPATCH(h->prec, st = hetero_solve<T>(h->d, h->hetero, 0.5 * (mmin + mmax), stress, stress ? sig : eps, tol,
+    FDM_DISPATCH(h->prec, st = hetero_solve<T>(h->d, h->hetero, mu0, stress, stress ? sig : eps, tol,
                                                max_iter, h->stream, &it, &r));
     if (st) return st;
     if (h->hetero_on) {   // the uploaded field replaces the stepping field
-        h->hetero_mu0 = 0.5 * (mmin + mmax);
+        h->hetero_mu0 = mu0;
         h->hetero_tol = tol;
         h->hetero_max_iter = max_iter;
     }
-    if (sigma13 && (st = download_field(sigma13, h->d.tau, n, h->prec, 0.0, h->stream))) return st;
-    if (sigma23 && (st = download_field(sigma23, h->hetero.t2, n, h->prec, 0.0, h->stream))) return st;
+    const Stage stage = state_stage(h->d, h->prec, 0, 1 - s.cur);
+    if (sigma13 && (st = download_field(sigma13, h->d.tau, n, h->prec, 0.0, stage, h->stream))) return st;
+    if (sigma23 && (st = download_field(sigma23, h->hetero.t2, n, h->prec, 0.0, stage, h->stream))) return st;
     FDM_CK(cudaStreamSynchronize(h->stream));
     if (iterations) *iterations = it;
     if (residual) *residual = r;
@@ -1003,7 +1094,7 @@ fdm_status fdm_set_mobility_field(fdm_handle* h, const double* factor) {
         fdm_status st = h->arena.alloc(&h->mfac_buf, h->n * elt_size(&h->d.p));
         if (st) return st;
     }
-    fdm_status st = upload_field(h->mfac_buf, factor, h->n, h->prec, 0.0, h->stream);
+    fdm_status st = upload_field(h->mfac_buf, factor, h->n, h->prec, 0.0, spectrum_stage(h->d, h->prec), h->stream);
     if (st) return st;
     h->d.mfac = h->mfac_buf;
     return FDM_OK;

@@ -182,9 +182,43 @@ struct Arena {
 template <typename T>
 fdm_status build_group(Dev& d, Arena& A, const fdm_params& p, int count, int gated, bool with_spec2, cudaStream_t s);
 
+// Host fields of at least this many values cross the link as doubles and are split, merged and
+// summed on the device (2048^2 with pinned arrays, one field set and two read: FP32 pairs 16.1 ->
+// 1.5 ms, double words 25 -> 1.1 ms); smaller ones are converted on the host on their way in, where
+// the launches and the wait for the sum would cost more than the loop.
+constexpr size_t kHostField = 16384;
+
+// Device space for doubles on their way: up to two pieces of a dead buffer.  FP64 and double-word
+// buffers of n values hold n doubles; a pair of FP32 buffers n / 2 each.
+struct Stage {
+    double* piece[2];
+    size_t len[2];
+};
+// state buffer b (not the current one) of instance inst: nothing reads it before the stencil has
+// written it, so it is free at any time between two kernels of a step
+Stage state_stage(const Dev& d, int prec, int inst, int b);
+// a host FP64 field to device doubles (in pieces), with its compensated sum, its largest magnitude
+// (NaN if any value is) and its least value where it is positive; waits
+struct FieldStats { double sum, top, low; };
+fdm_status stage_upload(const Stage& g, const double* src, double* red, double* red_host, int nblk, FieldStats* st,
+                        cudaStream_t s);
+// staged doubles minus offset to a field of precision `prec`
+fdm_status stage_convert(const Stage& g, void* dst, int prec, double offset, cudaStream_t s);
+
 // Uploads a host FP64 field into a device buffer of precision `prec` (FDM_FP64, FDM_MIXED,
-// FDM_DF64), minus offset / downloads it, adding offset back.
-fdm_status upload_field(void* dst, const double* src, size_t n, int prec, double offset, cudaStream_t s);
+// FDM_DF64), minus offset / downloads it, adding offset back, by way of the doubles of `stage`
+// (which may not be the field itself).
+fdm_status upload_field(void* dst, const double* src, size_t n, int prec, double offset, const Stage& stage,
+                        cudaStream_t s);
+fdm_status download_field(double* dst, const void* src, size_t n, int prec, double offset, const Stage& stage,
+                          cudaStream_t s);
+// Sets U13 of instance `inst` from host doubles (minus the mean for FDM_MIXED, which stores FP32
+// pairs hi = fl(v), lo = fl(v - hi), and FDM_DF64): the new state goes to buffer *cur (updated),
+// *mean receives the field's mean.  FDM_ERR_INVALID_ARG, and the old state kept, if that is not
+// finite.
+fdm_status set_state(const Dev& d, int prec, int inst, const double* src, int* cur, double* mean, cudaStream_t s);
+// U13 of instance `inst` in state buffer b, the current one, to host doubles (plus `offset`)
+fdm_status download_state(double* dst, const Dev& d, int prec, int b, int inst, double offset, cudaStream_t s);
 
 // Heterogeneous antiplane static problem (fdm_hetero.cu): device fields of type T, n each:
 // the shear modulus, the iterate g (two components) and two work fields; gam: the Green
@@ -208,12 +242,6 @@ fdm_status hetero_layer_solve(const Dev& d, const double* f_dev, double f0, bool
                               double tol, int max_iter, const int* planes_dev, int nplanes, double* tau_out,
                               double* planes_out, void* const bufs[3], double* partials, int nblk, cudaStream_t s,
                               int* iterations, double* residual);
-fdm_status download_field(double* dst, const void* src, size_t n, int prec, double offset, cudaStream_t s);
-// U13 of instance `inst` in state buffer b, from / to host doubles (minus / plus `offset`);
-// FDM_MIXED stores FP32 pairs: hi = fl(v), lo = fl(v - hi)
-fdm_status upload_state(const Dev& d, int prec, int b, int inst, const double* src, double offset, cudaStream_t s);
-fdm_status download_state(double* dst, const Dev& d, int prec, int b, int inst, double offset, cudaStream_t s);
-
 // A step of every group as CUDA graphs (1 and kGraphSteps steps), replayed on a stream.
 // Whole steps recorded as CUDA graphs.  With several groups each group's kernels form their
 // own branch of the graph (captured on a side stream forked from and joined back to the

@@ -107,6 +107,14 @@ template <typename T> void launch_alpha_sums(const Dev& d, int inst, double* par
 template <typename T>
 void launch_velocity(const Dev& d, const T* a11, const T* a12, const T* tau, const T* phi, T* v1, T* v2,
                      cudaStream_t s);
+// host fields: doubles to FP32 pairs of v - offset; (a or the pair a + lo) + offset as doubles;
+// f v in the field type; sums and extremes (4 doubles per block: sum, its error, the largest
+// magnitude, the least value of a positive field)
+void launch_split_pair(const double* src, float* hi, float* lo, size_t n, double offset, cudaStream_t s);
+template <typename T>
+void launch_merge(const T* a, const T* lo, double* out, size_t n, double offset, cudaStream_t s);
+template <typename T> void launch_scale(const double* a, T* b, size_t n, double f, cudaStream_t s);
+void launch_field_stats(const double* x, size_t n, double* partials, int nblk, cudaStream_t s);
 void launch_pair_to_double(const float* hi, const float* lo, double* out, size_t n, cudaStream_t s);
 // U13 of the current state (FP64) against prev[n]: partials[2 nblk] = per block sum of
 // (U - prev)^2 and of prev^2, then prev <- U; first = 1 only copies

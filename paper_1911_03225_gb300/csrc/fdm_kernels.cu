@@ -779,6 +779,87 @@ void launch_pair_to_double(const float* hi, const float* lo, double* out, size_t
     pair_to_double_kernel<<<4 * 152, 256, 0, s>>>(hi, lo, out, n);
 }
 
+// Host fields cross as doubles and are split or merged here: the FP32 pair of v - offset, or its
+// double word, and back.  Bound by the copy over the host link (measured beside the host loops
+// they replace: see kHostField in fdm_host.h).
+__global__ void split_pair_kernel(const double* __restrict__ src, float* __restrict__ hi, float* __restrict__ lo,
+                                  size_t n, double offset) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double v = src[i] - offset;
+        const float h = (float)v;
+        hi[i] = h;
+        lo[i] = (float)(v - (double)h);
+    }
+}
+void launch_split_pair(const double* src, float* hi, float* lo, size_t n, double offset, cudaStream_t s) {
+    split_pair_kernel<<<4 * 152, 256, 0, s>>>(src, hi, lo, n, offset);
+}
+template <typename T>
+__global__ void merge_kernel(const T* __restrict__ a, const T* __restrict__ lo, double* __restrict__ out, size_t n,
+                             double offset) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        out[i] = (lo ? (double)a[i] + (double)lo[i] : (double)a[i]) + offset;
+}
+template <typename T>
+void launch_merge(const T* a, const T* lo, double* out, size_t n, double offset, cudaStream_t s) {
+    merge_kernel<T><<<4 * 152, 256, 0, s>>>(a, lo, out, n, offset);
+}
+// per block: the sum of x as a double-word (sum, error) pair, and the largest and the smallest of
+// the values' keys (key 0: magnitude bits, a NaN above all; key 1: the value itself ordered as
+// signed bits, for positive fields)
+__global__ void field_stats_kernel(const double* __restrict__ x, size_t n, double* __restrict__ partials) {
+    __shared__ double rs[32], re[32];
+    __shared__ unsigned long long rmax[32];
+    __shared__ long long rmin[32];
+    double s = 0.0, e = 0.0;
+    unsigned long long top = 0ull;
+    long long low = 0x7fffffffffffffffll;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const double v = x[i];
+        neumaier_add(s, e, v);
+        const unsigned long long m = ubits(v) & kMagBits;
+        top = m > top ? m : top;
+        const long long k = __double_as_longlong(v);
+        low = k < low ? k : low;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+        neumaier_add(s, e, s2);
+        e += e2;
+        const unsigned long long t2 = __shfl_xor_sync(0xffffffffu, top, o);
+        top = t2 > top ? t2 : top;
+        const long long l2 = __shfl_xor_sync(0xffffffffu, low, o);
+        low = l2 < low ? l2 : low;
+    }
+    const int w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) { rs[w] = s; re[w] = e; rmax[w] = top; rmin[w] = low; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
+            neumaier_add(s, e, rs[i]);
+            e += re[i];
+            top = rmax[i] > top ? rmax[i] : top;
+            low = rmin[i] < low ? rmin[i] : low;
+        }
+        partials[4 * blockIdx.x] = s;
+        partials[4 * blockIdx.x + 1] = e;
+        partials[4 * blockIdx.x + 2] = dbits(top);
+        partials[4 * blockIdx.x + 3] = __longlong_as_double(low);
+    }
+}
+void launch_field_stats(const double* x, size_t n, double* partials, int nblk, cudaStream_t s) {
+    field_stats_kernel<<<nblk, 256, 0, s>>>(x, n, partials);
+}
+template <typename T>
+__global__ void scale_kernel(const double* __restrict__ a, T* __restrict__ b, size_t n, double f) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        b[i] = T(f * a[i]);
+}
+template <typename T> void launch_scale(const double* a, T* b, size_t n, double f, cudaStream_t s) {
+    scale_kernel<T><<<4 * 152, 256, 0, s>>>(a, b, n, f);
+}
+
 template <typename T>
 __global__ void convert_kernel(const double* __restrict__ a, T* __restrict__ b, size_t n, double offset) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -1560,6 +1641,8 @@ cudaError_t persist_launch(const void* dev_desc, int ngroups, int nsteps, Persis
                                      cudaStream_t);                                                     \
     template void launch_twiddle_tables<T>(void*, int, void*, int, cudaStream_t);                          \
     template void launch_state_change<T>(const Dev&, double*, int, double*, int, cudaStream_t);                          \
+    template void launch_merge<T>(const T*, const T*, double*, size_t, double, cudaStream_t);              \
+    template void launch_scale<T>(const double*, T*, size_t, double, cudaStream_t);                        \
     template void launch_fft_forward_many<T>(const Dev&, const T*, void*, int, cudaStream_t);              \
     template void launch_fft_inverse_many<T>(const Dev&, void*, T*, int, cudaStream_t);
 FDM_INST(double)
