@@ -66,13 +66,12 @@ fdm_status build_group(Dev& d, Arena& A, const fdm_params& p, int count, int gat
     if ((st = A.alloc((void**)&d.red, (size_t)6 * d.red_blocks * sizeof(double)))) return st;
     if ((st = A.alloc_host((void**)&d.red_host, kInfoScalarBytes + (size_t)6 * d.red_blocks * sizeof(double))))
         return st;
-    if ((st = A.alloc((void**)&d.sc, (size_t)count * sizeof(fdm_dev_scalars)))) return st;
-    FDM_CK(cudaMemsetAsync(d.sc, 0, (size_t)count * sizeof(fdm_dev_scalars), s));
-    if (!std::is_same<T, float>::value) {
-        const size_t chunk_bytes = (size_t)count * list_chunks(n) * sizeof(unsigned);
-        if ((st = A.alloc((void**)&d.chunks, chunk_bytes))) return st;
-        FDM_CK(cudaMemsetAsync(d.chunks, 0, chunk_bytes, s));
-    }
+    // the scalars and, behind them, the counters of the stencil's lists
+    const size_t sc_bytes = (size_t)count * sizeof(fdm_dev_scalars);
+    const size_t chunk_bytes = std::is_same<T, float>::value ? 0 : (size_t)count * list_chunks(n) * sizeof(unsigned);
+    if ((st = A.alloc((void**)&d.sc, sc_bytes + chunk_bytes))) return st;
+    if (chunk_bytes) d.chunks = (unsigned*)((char*)d.sc + sc_bytes);
+    FDM_CK(cudaMemsetAsync(d.sc, 0, sc_bytes + chunk_bytes, s));
     FDM_CK(cudaMemsetAsync(d.phi[0], 0, cn * sizeof(T), s));
     if ((st = upload_twiddles<T>(d.tw1, p.n1, s))) return st;
     if ((st = upload_twiddles<T>(d.tw2, p.n2, s))) return st;

@@ -369,12 +369,19 @@ __global__ void __launch_bounds__(FixBlock<L, false>::most, FixBlock<L, false>::
                 if (on && c == 0) {
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        // z = C0 + i CN: out(ky) = (m0 + mN)/2 z(ky) + (m0 - mN)/2 conj(z(-ky))
+                        // z = C0 + i CN: out(ky) = (m0 + mN)/2 z(ky) + (m0 - mN)/2 conj(z(-ky)),
+                        // the symbols real (K, some stress components) or imaginary
                         const int ky = j + u * T;
                         const cpx<double> m0 = col_multiplier<double>(a, Kh, 0, ky, n1, n2);
                         const cpx<double> mN = col_multiplier<double>(a, Kh, n1 / 2, ky, n1, n2);
-                        const cpx<double> zr = W[fix_pad((n2 - ky) & (n2 - 1))];
-                        x[u] = cmul(scale(m0 + mN, 0.5), x[u]) + cmul(scale(m0 - mN, 0.5), conj(zr));
+                        const cpx<double> z = x[u], zr = W[fix_pad((n2 - ky) & (n2 - 1))];
+                        if (a.mode == COL_K || (a.mode == COL_SYM && !a.sym_imag)) {
+                            const double p = 0.5 * (m0.x + mN.x), d = 0.5 * (m0.x - mN.x);
+                            x[u] = mk(p * z.x + d * zr.x, p * z.y - d * zr.y);
+                        } else {
+                            const double p = 0.5 * (m0.y + mN.y), d = 0.5 * (m0.y - mN.y);
+                            x[u] = mk(d * zr.y - p * z.y, p * z.x + d * zr.x);
+                        }
                         if (ky == 0 && a.mode == COL_K) x[u].x = 0.0;   // the macroscopic stress: see fix_row_inverse_kernel
                     }
                 }
@@ -545,6 +552,7 @@ __global__ void __launch_bounds__(FixBlock<L, true>::most, FixBlock<L, true>::mi
     else FIX_SWITCH(L, BODY)
 
 template <typename K> cudaError_t allow_smem(K* k, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;   // allowed as it is
     cudaError_t e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute((const void*)k, cudaFuncAttributePreferredSharedMemoryCarveout,

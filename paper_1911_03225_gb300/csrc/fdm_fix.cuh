@@ -188,16 +188,18 @@ FIX_HD double fix_from_bits(unsigned long long u) {
 }
 // the high word of |x| (its exponent above the top 20 mantissa bits)
 FIX_HD unsigned fix_mag(double x) { return (unsigned)(fix_bits(x) >> 32) & 0x7fffffffu; }
-// x in units of 2^(E - 1080), truncated toward zero; E >= kFixLowExp at least x's exponent
-FIX_HD long long fix_from(double x, int E) {
+// x in units of 2^(E - 1022 - B), truncated toward zero (or, NEAR, rounded to nearest); E >=
+// kFixLowExp at least x's exponent: |result| <= 2^B
+template <int B = kFixBits, bool NEAR = false> FIX_HD long long fix_from(double x, int E) {
     const unsigned long long u = fix_bits(x);
     const int d = E - ((int)(u >> 52) & 0x7ff);
-    unsigned long long m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 5;
+    unsigned long long m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << (B - 53 + (NEAR ? 1 : 0));
 #if defined(__CUDA_ARCH__)
     asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(d));   // 0 beyond 63
 #else
     m = d > 63 ? 0 : m >> d;
 #endif
+    if (NEAR) m = (m + 1) >> 1;
     const long long s = (long long)u >> 63;
     return ((long long)m ^ s) - s;
 }
@@ -281,6 +283,341 @@ FIX_HD void fix_c2r(cfx xk, cfx xc, twx w, cfx* zk, cfx* zc) {
     const cfx O = fix_mul<+1>(mkx(A.x - B.x, A.y - B.y), w, 1);
     *zk = mkx(E.x - O.y, E.y + O.x);
     *zc = mkx(E.x + O.y, O.x - E.y);
+}
+
+// ---------------------------------------------------------------------------------
+// The FP64 stencil's short node update (nodes of one characteristic direction, fdm_device.cuh) in
+// the same arithmetic.  The first
+// differences are FP64 subtractions; from there the node works in units of 2^(E - 1080) with E the
+// exponent of its largest difference, five bits below the last of that difference, rounded to
+// nearest (truncation would drift: 200 steps of two walls that annihilate, whose amplitude falls
+// by 42 decades, end 2.3e-15 from an 80-bit run against 4.0e-15 for FP64 arithmetic and 6.5e-15
+// with truncation).  Integer instructions and 13 FP64 ones per node replace 39 FP64 ones.
+// ---------------------------------------------------------------------------------
+// (a b) / 2^64 rounded (the product of the low halves left out), |a|, |b| <= 2^62 (fix_halves
+// rounds up: it needs 2^31 of room below 2^63)
+FIX_HD long long fix_mulhi(long long a, long long b) {
+    int ah, al, bh, bl;
+    fix_halves(a, ah, al);
+    fix_halves(b, bh, bl);
+    const long long q = fix_mad(al, bh, fix_mad(ah, bl, 0x80000000ll));
+    return fix_mad(fix_hi(q), 1, fix_wide(ah, bh));
+}
+// (a b) / 2^(64 - s)
+FIX_HD long long fix_mulhi(long long a, long long b, int s) {
+    int ah, al, bh, bl;
+    fix_halves(a, ah, al);
+    fix_halves(b, bh, bl);
+    const long long q = fix_mad(al, bh, fix_mad(ah, bl, (long long)(0x80000000u >> s)));
+    return fix_combine(fix_wide(ah, bh), q, s);
+}
+// (a b + c d) / 2^(64 - s)
+FIX_HD long long fix_mulhi2(long long a, long long b, long long c, long long d, int s) {
+    int ah, al, bh, bl, ch, cl, dh, dl;
+    fix_halves(a, ah, al);
+    fix_halves(b, bh, bl);
+    fix_halves(c, ch, cl);
+    fix_halves(d, dh, dl);
+    const long long t = fix_mad(ch, dh, fix_wide(ah, bh));
+    const long long q = fix_mad(cl, dh, fix_mad(ch, dl, fix_mad(al, bh, fix_mad(ah, bl, (long long)(0x80000000u >> s)))));
+    return fix_combine(t, q, s);
+}
+// of one sign and none zero: the one of least magnitude, else 0
+FIX_HD long long fix_minmod3(long long a, long long b, long long c) {
+    const long long s = a >> 63;
+    long long m = a ^ s;
+    const long long mb = b ^ s, mc = c ^ s;   // negative where the signs differ (or zero meets a negative)
+    m = mb < m ? mb : m;
+    m = mc < m ? mc : m;
+    return (m ^ s) & ~(m >> 63);
+}
+// the limiter parameter: code 1 or 2 when it is exactly that, else 2^-2 theta as fix_split's halves
+struct FixTheta { int code, h, l; };
+FIX_HD long long fix_theta(long long a, FixTheta t) {
+    if (t.code == 1) return a;
+    if (t.code == 2) return a + a;
+    int h, l;
+    fix_halves(a, h, l);
+    return fix_combine(fix_wide(h, t.h), fix_mad(l, t.h, fix_mad(h, t.l, 0x20000000ll)), 2);
+}
+FIX_HD int fix_clz(long long v) {   // v > 0
+#if defined(__CUDA_ARCH__)
+    return __clzll(v);
+#else
+    return __builtin_clzll((unsigned long long)v);
+#endif
+}
+FIX_HD float fix_rsqrt_seed(unsigned x) {   // 1 / sqrt(x), relative error below 2^-21
+#if defined(__CUDA_ARCH__)
+    return rsqrtf((float)x);
+#else
+    return 1.0f / __builtin_sqrtf((float)x) * (1.0f + 0x1p-22f);
+#endif
+}
+FIX_HD int fix_round(float v) {
+#if defined(__CUDA_ARCH__)
+    return __float2int_rn(v);
+#else
+    return (int)__builtin_rintf(v);
+#endif
+}
+// 2^61 / sqrt(x 2^-58) for x in [2^56, 2^59), relative error below 2^-56: the float seed y0 and
+// y0 (1 + e / 2 + 3 e^2 / 8) with e = 1 - x y0^2 (the binomial series; |e| < 2^-20)
+FIX_HD long long fix_rsqrt(long long x) {
+    const float s = fix_rsqrt_seed((unsigned)((unsigned long long)x >> 27)) * 0x1.6a09e6p15f;   // y0: x 2^-27 = xi 2^31
+    const int y = fix_round(s * 0x1p29f);                          // y0 2^29 in (2^28, 2^30]
+    const long long one = (long long)1 << 57;
+    const long long e = one - fix_mulhi(x << 3, fix_wide(y, y) << 2);   // 2^57 e
+    int eh, el;
+    fix_halves(e, eh, el);
+    // y0 e / 2 in units of 2^-61: y e 2^-26
+    const long long d = (fix_wide(y, eh) << 6) + (fix_wide(y, el) >> 26);
+    const float ef = (float)(int)(e >> 16) * 0x1p-41f;
+    const int c = fix_round(s * (0.375f * ef) * ef * 0x1p61f);
+    return fix_mad(c, 1, ((long long)y << 32) + d);
+}
+// (p, q) shifted left by *L so that the larger has 61 bits, and |(p, q)|^2 of those / 2^64, in
+// [2^56, 2^59); false for (0, 0)
+FIX_HD bool fix_norm2(long long p, long long q, long long* ps, long long* qs, int* L, long long* r2) {
+    const long long sp = p >> 63, sq = q >> 63;
+    const long long m = ((p ^ sp) - sp) | ((q ^ sq) - sq);
+    if (m == 0) return false;
+    *L = fix_clz(m) - 3;
+    *ps = (long long)((unsigned long long)p << *L);
+    *qs = (long long)((unsigned long long)q << *L);
+    int ph, pl, qh, ql;
+    fix_halves(*ps, ph, pl);
+    fix_halves(*qs, qh, ql);
+    const long long t = fix_mad(qh, qh, fix_wide(ph, ph));
+    const long long h = fix_mad(ql, qh, fix_mad(pl, ph, 0x40000000ll));   // half the cross terms
+    *r2 = t + (h >> 31);
+    return true;
+}
+
+// returns whether the node qualifies (and *out its new value); nodes whose scale lies
+// near the ends of FP64's range, or whose cross difference dwarfs the others, do not
+template <typename F>
+FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level, double* out) {
+    const double f0 = f(0, 0);
+    const double xm = f(-1, 0), xp = f(1, 0), ym = f(0, -1), yp = f(0, 1);
+    const double axm3 = xm - f(-2, 0), axm1 = f0 - xm, axp1 = xp - f0, axp3 = f(2, 0) - xp;
+    const double aym3 = ym - f(0, -2), aym1 = f0 - ym, ayp1 = yp - f0, ayp3 = f(0, 2) - yp;
+    auto top = [](unsigned a, unsigned b) { return a > b ? a : b; };
+    const unsigned m = top(top(top(fix_mag(axm3), fix_mag(axm1)), top(fix_mag(axp1), fix_mag(axp3))),
+                           top(top(fix_mag(aym3), fix_mag(aym1)), top(fix_mag(ayp1), fix_mag(ayp3))));
+    const int E = (int)(m >> 20);
+    if (E < kFixLowExp || E > kFixHighExp) {
+        if (m != 0u) return false;
+        const unsigned long long any = fix_bits(axm3) | fix_bits(axm1) | fix_bits(axp1) | fix_bits(axp3) |
+                                       fix_bits(aym3) | fix_bits(aym1) | fix_bits(ayp1) | fix_bits(ayp3);
+        *out = f0;   // no gradient: H = 0
+        return (any << 1) == 0ull;
+    }
+    const double vdt = v0 * dt_h;
+    if ((fix_mag(vdt) >> 20) > 1023u) return false;
+    const int Es = E + 1;   // |differences| < 2^58, the cross difference's below 2^59
+    const long long dxm3 = fix_from<59, true>(axm3, Es), dxm1 = fix_from<59, true>(axm1, Es), dxp1 = fix_from<59, true>(axp1, Es), dxp3 = fix_from<59, true>(axp3, Es);
+    const long long dym3 = fix_from<59, true>(aym3, Es), dym1 = fix_from<59, true>(aym1, Es), dyp1 = fix_from<59, true>(ayp1, Es), dyp3 = fix_from<59, true>(ayp3, Es);
+    const long long cxl = fix_theta(dxp1 - dxm1, th), cyl = fix_theta(dyp1 - dym1, th);
+    const long long Sx0 = fix_minmod3(fix_theta(dxp3 - dxp1, th), (dxp3 - dxm1) >> 1, cxl);
+    const long long Sx1 = fix_minmod3(cxl, (dxp1 - dxm3) >> 1, fix_theta(dxm1 - dxm3, th));
+    const long long Sy0 = fix_minmod3(fix_theta(dyp3 - dyp1, th), (dyp3 - dym1) >> 1, cyl);
+    const long long Sy1 = fix_minmod3(cyl, (dyp1 - dym3) >> 1, fix_theta(dym1 - dym3, th));
+    const long long px0 = dxp1 - (Sx0 >> 1), px1 = dxm1 + (Sx1 >> 1);
+    const long long qy0 = dyp1 - (Sy0 >> 1), qy1 = dym1 + (Sy1 >> 1);
+    const bool one_x = (px0 ^ px1) >= 0 && px0 != 0 && px1 != 0, one_y = (qy0 ^ qy1) >= 0 && qy0 != 0 && qy1 != 0;
+    const bool flat_x = (px0 | px1 | Sx0 | Sx1) == 0, flat_y = (qy0 | qy1 | Sy0 | Sy1) == 0;
+    if (!(one_x || flat_x) || !(one_y || flat_y)) return false;
+    // side 0 (+) where v0 and the derivative have opposite signs, side 1 (-) where they agree
+    const long long vs = (long long)fix_bits(v0);
+    const bool s0 = (vs ^ px0) < 0, t0 = (vs ^ qy0) < 0;
+    const int cx = s0 ? 1 : -1, cy = t0 ? 1 : -1;
+    const double fy = t0 ? yp : ym;
+    const double ac = f(cx, cy) - fy;
+    if ((int)(fix_mag(ac) >> 20) > Es) return false;
+    const long long fx = s0 ? dxp1 : -dxm1;
+    const long long mixed = fix_from<59, true>(ac, Es) - fx;
+    if (flat_x || flat_y) {
+        const double oc = flat_y ? f(cx, -cy) - (t0 ? ym : yp) : f(-cx, cy) - fy;   // the other quadrant's
+        if ((int)(fix_mag(oc) >> 20) > Es) return false;
+        if (mixed != 0 || fix_from<59, true>(oc, Es) != (flat_y ? fx : -fx)) return false;
+    }
+    const long long cross = (s0 == t0) ? mixed : -mixed;
+    const long long Sx = s0 ? Sx0 : Sx1, Sy = t0 ? Sy0 : Sy1;
+    long long p = s0 ? px0 : px1, q = t0 ? qy0 : qy1, ps, qs, r2;
+    int L;
+    if (time_level == 0 && fix_norm2(p, q, &ps, &qs, &L, &r2)) {
+        // (p, q) -= dt/2 Hess grad_(p,q) H, grad H = v0 (p, q) / |(p, q)|
+        const long long y = fix_rsqrt(r2);
+        const long long c = fix_mulhi(ps, y, 3), s = fix_mulhi(qs, y, 3);   // the direction, in units of 2^-61
+        const long long h = fix_from<kFixBits, true>(vdt, 1023) << 4;                        // v0 dt / (2 h) in units of 2^-62
+        p -= fix_mulhi(fix_mulhi2(Sx, c, cross, s, 3), h, 2);
+        q -= fix_mulhi(fix_mulhi2(cross, c, Sy, s, 3), h, 2);
+    }
+    double g = 0.0;   // h |grad|
+    if (fix_norm2(p, q, &ps, &qs, &L, &r2)) {
+        // |(p 2^L, q 2^L)| = 2^61 sqrt(xi), xi = r2 2^-58, sqrt(xi) = xi / sqrt(xi)
+        const long long r = fix_mulhi(r2 << 3, fix_rsqrt(r2));   // 2^58 sqrt(xi)
+        g = fix_to(r, Es - 1081 + 3 - L);
+    }
+    *out = f0 - vdt * g;
+    return true;
+}
+
+FIX_HD float fix_rcp_seed(float x) {   // 1 / x, relative error below 2^-21
+#if defined(__CUDA_ARCH__)
+    return __fdividef(1.0f, x);
+#else
+    return 1.0f / x * (1.0f - 0x1p-22f);
+#endif
+}
+// a / w in units of 2^-61, 0 <= a <= w, 0 < w <= 2^62 (2^-58 absolute): the reciprocal of w scaled
+// to [1/2, 1) from the float seed y0 as y0 (1 + e + e^2), e = 1 - w y0 (the geometric series)
+FIX_HD long long fix_ratio(long long a, long long w) {
+    const int L = fix_clz(w) - 1;
+    const long long wn = (long long)((unsigned long long)w << L) >> 2, an = (long long)((unsigned long long)a << L) >> 2;
+    const float s = fix_rcp_seed((float)(unsigned)((unsigned long long)wn >> 29) * 0x1p-32f);
+    const int y = fix_round(s * 0x1p29f);
+    const long long one = (long long)1 << 58;
+    const long long e = one - fix_mulhi(wn, (long long)y << 32);   // 2^58 e, wn = 2^61 w
+    int eh, el;
+    fix_halves(e, eh, el);
+    const float ef = (float)(int)(e >> 16) * 0x1p-42f;
+    const long long r = fix_mad(fix_round(s * ef * ef * 0x1p60f), 1,
+                                ((long long)y << 31) + (fix_wide(y, eh) << 5) + (fix_wide(y, el) >> 27));
+    return fix_mulhi(an, r, 4);
+}
+// |(p, q)| of integers in a node's units (0 for (0, 0))
+FIX_HD long long fix_norm(long long p, long long q) {
+    long long ps, qs, r2;
+    int L;
+    if (!fix_norm2(p, q, &ps, &qs, &L, &r2)) return 0;
+    const long long r = fix_mulhi(r2 << 3, fix_rsqrt(r2)) << 3;
+    return (r + ((1ll << L) >> 1)) >> L;
+}
+// (p, q) / |(p, q)| in units of 2^-61 ((0, 0) for (0, 0))
+FIX_HD void fix_direction(long long p, long long q, long long* c, long long* s) {
+    long long ps, qs, r2;
+    int L;
+    *c = *s = 0;
+    if (!fix_norm2(p, q, &ps, &qs, &L, &r2)) return;
+    const long long y = fix_rsqrt(r2);
+    *c = fix_mulhi(ps, y, 3);
+    *s = fix_mulhi(qs, y, 3);
+}
+
+// The whole scheme for one FP64 node (Sec. 3.2.3 Steps 1-4, readings G1-G7) in cell units and
+// fixed point: the units of fix_upwind with E over all twelve differences.  The update is homogeneous in
+// U13, so a node near the ends of FP64's range is updated at 2^+-600 times its values; one with a
+// NaN, an infinity or a displacement beyond two cells (no finite step has one) gets a NaN.
+template <typename F>
+FIX_HD double fix_node(F f, double v0, double dt_h, FixTheta th, int time_level) {
+    auto top = [](unsigned a, unsigned b) { return a > b ? a : b; };
+    double k = 1.0, back = 1.0;
+    double a[12];
+    int E;
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        auto g = [&](int i, int j) { return pass ? f(i, j) * k : f(i, j); };
+        const double f0 = g(0, 0), xm = g(-1, 0), xp = g(1, 0), ym = g(0, -1), yp = g(0, 1);
+        a[0] = xm - g(-2, 0);
+        a[1] = f0 - xm;
+        a[2] = xp - f0;
+        a[3] = g(2, 0) - xp;
+        a[4] = ym - g(0, -2);
+        a[5] = f0 - ym;
+        a[6] = yp - f0;
+        a[7] = g(0, 2) - yp;
+        a[8] = g(1, 1) - yp;     // the quadrants' differences f(cx, cy) - f(0, cy)
+        a[9] = g(1, -1) - ym;
+        a[10] = g(-1, 1) - yp;
+        a[11] = g(-1, -1) - ym;
+        unsigned m = 0;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) m = top(m, fix_mag(a[i]));
+        E = (int)(m >> 20);
+        if (pass || (E >= kFixLowExp && E <= kFixHighExp)) break;
+        const bool up = E < kFixLowExp;
+        k = up ? 0x1p600 : 0x1p-600;
+        back = up ? 0x1p-600 : 0x1p600;
+    }
+    const double vdt = v0 * dt_h;
+    if (E >= 0x7ff || (fix_mag(vdt) >> 20) > 1023u) return fix_from_bits(0x7ff8000000000000ull);
+    if (E < kFixLowExp) return f(0, 0);   // no difference, however scaled
+    const int Es = E;   // |differences| < 2^58
+    // Step 1
+    long long D[2][2], S[2][2], P[2][2];   // axis; side 0: +, 1: -
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const long long m3 = fix_from<kFixBits, true>(a[4 * x], Es), m1 = fix_from<kFixBits, true>(a[4 * x + 1], Es), p1 = fix_from<kFixBits, true>(a[4 * x + 2], Es),
+                        p3 = fix_from<kFixBits, true>(a[4 * x + 3], Es);
+        const long long c = fix_theta(p1 - m1, th);
+        D[x][0] = p1;
+        D[x][1] = m1;
+        S[x][0] = fix_minmod3(fix_theta(p3 - p1, th), (p3 - m1) >> 1, c);
+        S[x][1] = fix_minmod3(c, (p1 - m3) >> 1, fix_theta(m1 - m3, th));
+        P[x][0] = p1 - (S[x][0] >> 1);
+        P[x][1] = m1 + (S[x][1] >> 1);
+    }
+    // Step 2: the one-sided displacements v0 dt dH/d(p, q) in units of 2^-61, from the three pairs
+    // that attain their extremes: |p| / |(p, q)| falls as |q| grows, so those of dH/dp belong to
+    // the q of least magnitude, those of dH/dq to the p of least magnitude
+    auto mag = [](long long v) { return v ^ (v >> 63); };
+    const bool tq = mag(P[1][1]) < mag(P[1][0]), tp = mag(P[0][1]) < mag(P[0][0]);
+    const long long qm = tq ? P[1][1] : P[1][0], qo = tq ? P[1][0] : P[1][1], pm = tp ? P[0][1] : P[0][0];
+    const long long h = fix_from<kFixBits, true>(vdt, 1023) << 4;   // v0 dt / h in units of 2^-61
+    long long c0, c1, cc, s0, s1, so;
+    fix_direction(P[0][0], qm, &c0, &s0);
+    fix_direction(P[0][1], qm, &c1, &s1);
+    fix_direction(pm, qo, &cc, &so);
+    const long long e[2][2] = {{fix_mulhi(c0, h, 3), fix_mulhi(c1, h, 3)}, {fix_mulhi(tp ? s1 : s0, h, 3), fix_mulhi(so, h, 3)}};
+    long long d[2][2], w[2][2];   // displacements and weights of each axis's sides
+    const long long one = (long long)1 << 61;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const long long hi = e[x][0] > e[x][1] ? e[x][0] : e[x][1], lo = e[x][0] < e[x][1] ? e[x][0] : e[x][1];
+        d[x][0] = hi > 0 ? hi : 0;
+        d[x][1] = lo < 0 ? lo : 0;
+        const long long span = d[x][0] - d[x][1];
+        w[x][1] = span > 0 ? fix_ratio(d[x][0], span) : one >> 1;
+        w[x][0] = one - w[x][1];
+    }
+    // Step 3: along each axis X(e) = e (D + S (e + sg) / 2) and its derivative D + S (e + sg / 2)
+    long long X[2][2], dX[2][2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const long long sg = s == 0 ? -one : one;
+            X[x][s] = fix_mulhi(D[x][s] + fix_mulhi(S[x][s] >> 1, d[x][s] + sg, 3), d[x][s], 3);
+            dX[x][s] = D[x][s] + fix_mulhi(S[x][s], d[x][s] + (sg >> 1), 3);
+        }
+    long long acc = 0;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        if (w[0][s] == 0) continue;
+        long long accs = 0;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            if (w[1][t] == 0) continue;
+            const long long mixed = fix_from<kFixBits, true>(a[8 + 2 * s + t], Es) - (s == 0 ? D[0][0] : -D[0][1]);
+            const long long cross = (s == t) ? mixed : -mixed;
+            const long long cx = fix_mulhi(cross, d[0][s], 3);
+            const long long val = X[0][s] + X[1][t] + fix_mulhi(cx, d[1][t], 3);
+            long long p = dX[0][s] + fix_mulhi(cross, d[1][t], 3), q = dX[1][t] + cx;
+            if (time_level == 0) {
+                // (p, q) -= dt/2 Hess grad_(p,q) H, grad H = v0 (p, q) / |(p, q)|
+                long long c, n;
+                fix_direction(p, q, &c, &n);
+                p -= fix_mulhi(fix_mulhi2(S[0][s], c, cross, n, 3), h, 2);
+                q -= fix_mulhi(fix_mulhi2(cross, c, S[1][t], n, 3), h, 2);
+            }
+            const long long psi = val - fix_mulhi(fix_norm(p, q), h, 3);
+            accs += fix_mulhi(psi, w[1][t], 3);
+        }
+        acc += fix_mulhi(accs, w[0][s], 3);   // Step 4
+    }
+    return f(0, 0) + fix_to(acc, Es - 1080) * back;
 }
 
 }  // namespace fdm

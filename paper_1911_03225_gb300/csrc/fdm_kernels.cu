@@ -14,6 +14,7 @@
 // multiply by K, inverse FFT along x2) -> row_inverse (C2R, tau and max|v0|) -> knp_step.
 #include <type_traits>
 
+#include "fdm_fix.cuh"
 #include "fdm_step.cuh"
 
 namespace fdm {
@@ -379,10 +380,10 @@ struct KnpArgs {
     const T* lo1;
     T theta;
     int theta_code;          // 1 or 2 when theta is exactly that (exact scaling), else 0
+    FixTheta theta_fix;      // the same in fixed point (FP64)
     int time_level;
     fdm_dev_scalars* sc;     // scalars of instance 0
     int gated;
-    int gather;              // collect the warps' left-over nodes in the instances' lists
     unsigned* list;          // instance 0's list (y n1 + x); the next one list_stride on
     size_t list_stride;
     unsigned* chunks;        // entries in each chunk of instance 0's list; the next chunk_stride on
@@ -408,21 +409,25 @@ template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed 
 
 // grid (n1 / tx, n2 / (ty npt), instances); block (tx, ty); thread (i, j) updates the
 // nodes (bx + i, by + j + k ty), k < npt.  FP64 and double words: first the nodes that have one
-// characteristic direction (knp_upwind), nearly all of them on the fields the method meets; each
-// warp lists its others and works through them with the whole scheme (knp_node), 32 (or 64) at a
+// characteristic direction (fix_upwind, knp_upwind_df2), nearly all of them on the fields the method meets; each
+// warp lists its others and works through them with the whole scheme (fix_node,
+// knp_node_df2), 32 (or 64) at a
 // time.  What is left over, seldom a full warp's worth, goes on the instance's list in global
 // memory when the launch has several waves of blocks (the list lies in the spectrum's buffer,
 // free between the inverse row kernel and the next step's forward one): the warp that completes
 // a chunk of 32 (64) of the list works through it, and the instance's last block takes the rest.
 // On a launch that the GPU holds at once there are idle lanes to spare, and a tail would cost a
-// scheme's latency (25 us in FP64): each warp sees to its own.  No barrier follows the tile's
+// scheme's latency: each warp sees to its own, and double words take the whole scheme throughout
+// (128^2: 16 us against 20 for one form after the other).  No barrier follows the tile's
 // loads, so warps at the whole scheme and warps at the short one share the pipes.  A node's
 // result depends on the node alone, not on the lists.  2048^2, random field after 30 steps: FP64
-// 1388 -> 624 us, double words 348 -> 245 us (one list per block, behind a barrier: 733 and 369;
-// per warp only: 759 and 426).
+// 1388 -> 221 us (624 with the short form in FP64 arithmetic), double words 348 -> 209 us (lists
+// per block, behind a barrier: 733 and 369; per warp only: 759 and 426).  What bounds the FP64
+// kernel now is instruction issue: 54% of the slots, the integer pipe 57% and the FP64 pipe 49%
+// busy.
 // body of one block: the tile (tbx, tby) of instance inst, ntiles tiles per instance (the
 // last to start advances the clock); thread (tx_, ty_) of a tx x TY block
-template <typename T, int V>
+template <typename T, int V, bool GATHER>
 __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, const T* __restrict__ tau0, int n1, int n2,
                                               int npt, KnpArgs<T> a, int tbx, int tby, int inst, int ntiles, int tx_,
                                               int ty_, int tx) {
@@ -540,6 +545,25 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 lo_out[(size_t)yb * n1 + x] = lo;
             }
         }
+    } else if constexpr (std::is_same<T, df>::value && !GATHER) {
+        // double words on a small launch: the whole scheme for every node, two at once in the
+        // lanes of the packed FP32 instructions, an odd last one paired with itself and written once
+#pragma unroll 1
+        for (int k = 0; k < npt; k += 2) {
+            const int k2 = (k + 1 < npt) ? k + 1 : k;
+            const int ya = by + ty_ + k * TY, yb = by + ty_ + k2 * TY;
+            const int la = ty_ + k * TY + 2, lb = ty_ + k2 * TY + 2;
+            T va = celerity(a.vel, s_tau[la - 2][tx_], tile[la][lx], phi_ref);
+            T vb = celerity(a.vel, s_tau[lb - 2][tx_], tile[lb][lx], phi_ref);
+            if (a.vel.mfac) {
+                va = va * a.vel.mfac[inst * nn + (size_t)ya * n1 + x];
+                vb = vb * a.vel.mfac[inst * nn + (size_t)yb * n1 + x];
+            }
+            auto f = [&](int i, int j) -> df2 { return mkdf2(tile[la + j][lx + i], tile[lb + j][lx + i]); };
+            const df2 res = knp_node_df2(f, mkdf2(va, vb), dt, a.theta, a.theta_code, a.time_level);
+            out[(size_t)ya * n1 + x] = lane(res, 0);
+            if (k2 != k) out[(size_t)yb * n1 + x] = lane(res, 1);
+        }
     } else {
         unsigned short* list = s_list[tid >> 5];
         const unsigned below = (1u << (tid & 31)) - 1u;
@@ -583,8 +607,8 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 auto f = [&](int i, int j) -> T { return tile[ly + j][lx + i]; };
                 const size_t o = place(r, tx_);
                 T res;
-                const bool ok = knp_upwind(f, velocity(o, s_tau[r][tx_], tile[ly][lx]), dt, a.theta, a.theta_code,
-                                           a.time_level, &res);
+                const bool ok = fix_upwind(f, velocity(o, s_tau[r][tx_], tile[ly][lx]), dt, a.theta_fix, a.time_level,
+                                           &res);
                 if (ok) out[o] = res;
                 defer(!ok, r);
             }
@@ -594,7 +618,7 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
         unsigned* glist = a.list + inst * a.list_stride;
         unsigned* chunks = a.chunks + inst * a.chunk_stride;
         // own: the first nodes of the warp's list, in rounds; the rest joins the instance's list
-        const int own = a.gather ? count / kRound * kRound : count, rest = count - own;
+        const int own = GATHER ? count / kRound * kRound : count, rest = count - own;
         int done = 0;                  // of the warp's own
         int todo[2] = {-1, -1};        // chunks of the instance's list this warp completed
         int tail = 0, tail_chunk = 0;  // the instance's last block: entries of the unfinished chunk
@@ -628,7 +652,7 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
             if (done < own) m = min(kRound, own - done);
             else if (todo[0] >= 0) { c = todo[0]; todo[0] = -1; m = kRound; }
             else if (todo[1] >= 0) { c = todo[1]; todo[1] = -1; m = kRound; }
-            else if (!ended && a.gather) {
+            else if (GATHER && !ended) {
                 ended = true;
                 if (ln == 0) {
                     __threadfence();
@@ -651,27 +675,33 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 c = tail_chunk;
                 m = tail;
             } else break;
-            auto node = [&](int i, int* x, int* y) {
+            // the round's values: the tile (own nodes) or the field, by one generic address
+            const T* u = c < 0 ? &tile[2][2] : phi;
+            const T* st = c < 0 ? &s_tau[0][0] : tau;
+            const int pitch = c < 0 ? TX + 4 : n1, tpitch = c < 0 ? TX : n1;
+            const int mx = c < 0 ? -1 : n1 - 1, my = c < 0 ? -1 : n2 - 1;
+            auto node = [&](int i, int* x, int* y) {   // of the tile or of the field
                 if (c < 0) {
                     const int e = list[done + i];
-                    *x = bx + e % TX;
-                    *y = by + e / TX;
+                    *x = e % TX;
+                    *y = e / TX;
                 } else {
                     const unsigned k = __ldcg(glist + (size_t)c * kRound + i);
                     *x = (int)(k & (unsigned)(n1 - 1));
                     *y = (int)(k / (unsigned)n1);
                 }
             };
-            const int mx = n1 - 1, my = n2 - 1;
-            auto at = [&](int x, int y, int i, int j) -> T { return phi[(size_t)((y + j) & my) * n1 + ((x + i) & mx)]; };
+            auto at = [&](int x, int y, int i, int j) -> T { return u[((y + j) & my) * pitch + ((x + i) & mx)]; };
+            auto where = [&](int x, int y) -> size_t { return c < 0 ? place(y, x) : (size_t)y * n1 + x; };
             if constexpr (kTwo) {
                 if (2 * ln < m) {
                     int xa, ya, xb, yb;
                     node(2 * ln, &xa, &ya);
                     node(2 * ln + 1 < m ? 2 * ln + 1 : 2 * ln, &xb, &yb);
-                    const size_t oa = (size_t)ya * n1 + xa, ob = (size_t)yb * n1 + xb;
+                    const size_t oa = where(xa, ya), ob = where(xb, yb);
                     auto f = [&](int i, int j) -> df2 { return mkdf2(at(xa, ya, i, j), at(xb, yb, i, j)); };
-                    const df2 v0 = mkdf2(velocity(oa, tau[oa], phi[oa]), velocity(ob, tau[ob], phi[ob]));
+                    const df2 v0 = mkdf2(velocity(oa, st[ya * tpitch + xa], at(xa, ya, 0, 0)),
+                                         velocity(ob, st[yb * tpitch + xb], at(xb, yb, 0, 0)));
                     const df2 res = knp_node_df2(f, v0, dt, a.theta, a.theta_code, a.time_level);
                     out[oa] = lane(res, 0);
                     if (ob != oa) out[ob] = lane(res, 1);
@@ -680,9 +710,9 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 if (ln < m) {
                     int x, y;
                     node(ln, &x, &y);
-                    const size_t o = (size_t)y * n1 + x;
+                    const size_t o = where(x, y);
                     auto f = [&](int i, int j) -> T { return at(x, y, i, j); };
-                    out[o] = knp_node<T>(f, velocity(o, tau[o], phi[o]), dt, a.theta, a.theta_code, a.time_level);
+                    out[o] = fix_node(f, velocity(o, st[y * tpitch + x], f(0, 0)), dt, a.theta_fix, a.time_level);
                 }
             }
             if (c < 0) done += m;
@@ -690,11 +720,21 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
     }
 }
 
-template <typename T, int V>
-__global__ void __launch_bounds__(TX * KnpShapes<T>::ty[V], KnpShapes<T>::minb[V])
+// Blocks per SM the kernel is compiled for: the shape's own figure in FP32; four of 256 threads (64
+// registers, some spilled) in FP64, whose forms wait on long integer chains (2048^2 random field:
+// 327 us with two, 272 with three, 241 with four, 238 with five); in double words four for the
+// tallest tiles, which large grids take (2048^2: 247, 215 and 209 us with two, three and four), and
+// the shape's figure for the others (512^2: 33 us with two, 46 with four)
+template <typename T, int V, bool GATHER> constexpr int knp_blocks() {
+    if (std::is_same<T, float>::value || KnpShapes<T>::ty[V] != 8) return KnpShapes<T>::minb[V];
+    return std::is_same<T, double>::value || (GATHER && KnpShapes<T>::npt[V] == 4) ? 4 : KnpShapes<T>::minb[V];
+}
+
+template <typename T, int V, bool GATHER>
+__global__ void __launch_bounds__(TX * KnpShapes<T>::ty[V], knp_blocks<T, V, GATHER>())
     knp_step_kernel(const T* phi0, const T* phi1, const T* __restrict__ tau0, int n1, int n2, int npt,
                     KnpArgs<T> a) {
-    knp_step_body<T, V>(phi0, phi1, tau0, n1, n2, npt, a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x * gridDim.y,
+    knp_step_body<T, V, GATHER>(phi0, phi1, tau0, n1, n2, npt, a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x * gridDim.y,
                         threadIdx.x, threadIdx.y, blockDim.x);
 }
 
@@ -1199,16 +1239,24 @@ void launch_row_inverse(const Dev& d, const cpx<T>* spec, T* dst, int mode, doub
 }
 
 template <typename T, int V>
-void launch_knp_shape(const Dev& d, KnpArgs<T> a, cudaStream_t s) {
+void launch_knp_shape(const Dev& d, const KnpArgs<T>& a, cudaStream_t s) {
     constexpr int TY = KnpShapes<T>::ty[V];
     const int tx = d.p.n1 < TX ? d.p.n1 : TX;
     int npt = KnpShapes<T>::npt[V];
     while (npt > 1 && d.p.n2 < TY * npt) npt >>= 1;
     dim3 grid(d.p.n1 / tx, d.p.n2 / (TY * npt), d.count), block(tx, TY);
-    // two blocks of 256 threads to an SM: several waves from here on
-    a.gather = (size_t)grid.x * grid.y * grid.z * tx * TY > (size_t)2 * 152 * 2 * 256 ? 1 : 0;
-    knp_step_kernel<T, V><<<grid, block, 0, s>>>((const T*)d.phi[0], (const T*)d.phi[1], (const T*)d.tau,
-                                                 d.p.n1, d.p.n2, npt, a);
+    // lists (knp_step_body) from the size at which a launch takes several waves of blocks, counted
+    // at two blocks of 256 threads per SM
+    const bool gather = (size_t)grid.x * grid.y * grid.z * tx * TY > (size_t)2 * 152 * 2 * 256;
+    if constexpr (!std::is_same<T, float>::value) {
+        if (gather) {
+            knp_step_kernel<T, V, true><<<grid, block, 0, s>>>((const T*)d.phi[0], (const T*)d.phi[1], (const T*)d.tau,
+                                                               d.p.n1, d.p.n2, npt, a);
+            return;
+        }
+    }
+    knp_step_kernel<T, V, false><<<grid, block, 0, s>>>((const T*)d.phi[0], (const T*)d.phi[1], (const T*)d.tau,
+                                                        d.p.n1, d.p.n2, npt, a);
 }
 
 template <typename T>
@@ -1219,11 +1267,12 @@ KnpArgs<T> knp_args(const Dev& d) {
     a.lo1 = (const T*)d.phi_lo[1];
     a.theta = T(d.p.theta);
     a.theta_code = d.p.theta == 1.0 ? 1 : (d.p.theta == 2.0 ? 2 : 0);
+    a.theta_fix.code = a.theta_code;
+    fix_split(0.25 * d.p.theta, &a.theta_fix.h, &a.theta_fix.l);
     a.time_level = d.p.time_level;
     a.sc = d.sc;
     a.gated = d.gated;
     const size_t n = (size_t)d.p.n1 * d.p.n2;
-    a.gather = 0;   // set with the grid
     a.list = static_cast<unsigned*>(d.spec);
     a.list_stride = n * sizeof(T) / sizeof(unsigned);
     a.chunks = d.chunks;
@@ -1529,7 +1578,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
                     } else if (phase == 2) {
                         row_inverse_body<float>(G.spec, G.tau, G.n1, G.n2, G.R, G.tw1, G.pt1, G.row, tile, inst, per);
                     } else {
-                        knp_step_body<float, kPersistShape>(G.phi0, G.phi1, G.tau, G.n1, G.n2, G.knp_npt, G.knp,
+                        knp_step_body<float, kPersistShape, false>(G.phi0, G.phi1, G.tau, G.n1, G.n2, G.knp_npt, G.knp,
                                                             tile % G.knp_gx, tile / G.knp_gx, inst, per,
                                                             threadIdx.x & (TX - 1), threadIdx.x / TX, TX);
                     }
