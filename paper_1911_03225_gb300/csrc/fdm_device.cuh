@@ -228,6 +228,28 @@ __device__ void smem_fft_ip(cpx<T>* a, int L, int nseq, int ld, const cpx<T>* __
 __device__ __forceinline__ float thalf(float x);
 template <typename T> __device__ __forceinline__ cpx<T> chalf(cpx<T> a) { return mk(thalf(a.x), thalf(a.y)); }
 
+template <typename T> struct cpair { cpx<T> a, b; };
+// X(k) and X(L - k) from A = Z(k) and B = conj Z(L - k)
+template <typename T> __device__ __forceinline__ cpair<T> r2c_pair(cpx<T> A, cpx<T> B, cpx<T> w) {
+    cpx<T> E = chalf(A + B);
+    cpx<T> D = chalf(A - B);
+    cpx<T> O = mk(D.y, -D.x);          // -i (A - B) / 2
+    cpx<T> WO = cmul(w, O);
+    cpair<T> r;
+    r.a = E + WO;
+    r.b = conj(E - WO);
+    return r;
+}
+// Z(k) and Z(L - k) from Xk = X(k), Xc = conj X(L - k) and v = exp(+2 pi i k / n)
+template <typename T> __device__ __forceinline__ cpair<T> c2r_pair(cpx<T> Xk, cpx<T> Xc, cpx<T> v) {
+    cpx<T> E = Xk + Xc;
+    cpx<T> O = cmul(Xk - Xc, v);
+    cpair<T> r;
+    r.a = mk(E.x - O.y, E.y + O.x);    // E + i O
+    r.b = mk(E.x + O.y, -E.y + O.x);   // conj(E) + i conj(O)
+    return r;
+}
+
 template <typename T>
 __device__ __forceinline__ void r2c_twist_pair(const cpx<T>* Z, cpx<T>* P, int L, int k,
                                                const cpx<T>* __restrict__ tw_n) {
@@ -236,13 +258,9 @@ __device__ __forceinline__ void r2c_twist_pair(const cpx<T>* Z, cpx<T>* P, int L
         P[0] = mk(z0.x + z0.y, z0.x - z0.y);
         return;
     }
-    cpx<T> A = Z[swz(k)], B = conj(Z[swz(L - k)]);
-    cpx<T> E = chalf(A + B);
-    cpx<T> D = chalf(A - B);
-    cpx<T> O = mk(D.y, -D.x);          // -i (A - B) / 2
-    cpx<T> WO = cmul(tw_n[k], O);
-    P[swz(k)] = E + WO;
-    if (2 * k != L) P[swz(L - k)] = conj(E - WO);
+    const cpair<T> r = r2c_pair(Z[swz(k)], conj(Z[swz(L - k)]), tw_n[k]);
+    P[swz(k)] = r.a;
+    if (2 * k != L) P[swz(L - k)] = r.b;
 }
 
 template <typename T>
@@ -253,11 +271,9 @@ __device__ __forceinline__ void c2r_twist_pair(const cpx<T>* P, cpx<T>* Z, int L
         Z[0] = mk(p0.x + p0.y, p0.x - p0.y);
         return;
     }
-    cpx<T> Xk = P[swz(k)], Xc = conj(P[swz(L - k)]);
-    cpx<T> E = Xk + Xc;
-    cpx<T> O = cmul(Xk - Xc, conj(tw_n[k]));  // times V^k = exp(+2 pi i k / n)
-    Z[swz(k)] = mk(E.x - O.y, E.y + O.x);          // E + i O
-    if (2 * k != L) Z[swz(L - k)] = mk(E.x + O.y, -E.y + O.x);  // conj(E) + i conj(O)
+    const cpair<T> r = c2r_pair(P[swz(k)], conj(P[swz(L - k)]), conj(tw_n[k]));
+    Z[swz(k)] = r.a;
+    if (2 * k != L) Z[swz(L - k)] = r.b;
 }
 
 // ---------------------------------------------------------------------------------

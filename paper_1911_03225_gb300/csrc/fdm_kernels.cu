@@ -169,8 +169,6 @@ __device__ __forceinline__ void col_pass_body(const cpx<T>* in, cpx<T>* out, int
     const size_t half_n = (size_t)n1 * n2 / 2;
     in += inst * half_n;
     out += inst * half_n;
-    fdm_dev_scalars* sci = a.sc ? a.sc + inst : nullptr;
-    const double* parts = a.row_partials ? a.row_partials + (size_t)inst * a.nparts : nullptr;
     const int kx0 = tile * C;
     const cpx<T>* src = in + (size_t)kx0 * n2;
     {
@@ -178,32 +176,7 @@ __device__ __forceinline__ void col_pass_body(const cpx<T>* in, cpx<T>* out, int
         for (int e = threadIdx.x; e < total; e += step) copy_async(A + (e >> ln2) * ld + swz(e & (n2 - 1)), src + e);
         copy_async_wait_all();
     }
-    if (a.mode == COL_K && kx0 == 0) {
-        // <U13> from the row sums, then the loading state of this step (Sec. 5.1).  The
-        // order is fixed by n2 alone: kRedLanes compensated lane sums over a stride, then a
-        // fixed tree (results do not depend on the launch shape)
-        for (int v = threadIdx.x; v < kRedLanes; v += blockDim.x) {
-            double s = 0.0, c = 0.0;
-            for (int i = v; parts && i < a.nparts; i += kRedLanes) neumaier_add(s, c, parts[i]);
-            s_red[v] = s + c;
-        }
-        __syncthreads();
-        double tot = 0.0;
-        if (threadIdx.x < 32) {
-            double s = 0.0, c = 0.0;
-            for (int v = threadIdx.x; v < kRedLanes; v += 32) neumaier_add(s, c, s_red[v]);
-            tot = warp_sum(s + c);
-        }
-        if (threadIdx.x == 0) {
-            double mean = parts ? sci->phi_ref + tot / ((double)n1 * (double)n2) : sci->mean_up13;
-            double eps, sig;
-            loading_state(a.p, sci->step, sci->t, mean, &eps, &sig);
-            sci->mean_up13 = mean;
-            sci->eps_bar13 = eps;
-            sci->sigma_bar13 = sig;
-            s_sigma = sig;
-        }
-    }
+    if (a.mode == COL_K && kx0 == 0) loading_from_rows(a, n1, n2, inst, s_red, &s_sigma);
     __syncthreads();
     cpx<T>* F = A;
     if (a.mode != COL_INV) F = block_fft<-1>(A, B, n2, C, ld, ptw);
@@ -222,15 +195,8 @@ __device__ __forceinline__ void col_pass_body(const cpx<T>* in, cpx<T>* out, int
                 o = col_apply<T>(a, Kh, kx, ky, n1, n2, z);
                 orr = col_apply<T>(a, Kh, kx, kyr, n1, n2, zr);
             } else {
-                // packed column: z = C0 + i CN (C0, CN transforms of the real columns kx = 0
-                // and kx = n1/2); multiply each by its own symbol and repack:
-                // out(ky) = (m0 + mN)/2 z(ky) + (m0 - mN)/2 conj(z(-ky))
-                cpx<T> m0 = col_multiplier<T>(a, Kh, 0, ky, n1, n2);
-                cpx<T> mN = col_multiplier<T>(a, Kh, n1 / 2, ky, n1, n2);
-                o = cmul(scale(m0 + mN, T(0.5)), z) + cmul(scale(m0 - mN, T(0.5)), conj(zr));
-                cpx<T> m0r = col_multiplier<T>(a, Kh, 0, kyr, n1, n2);
-                cpx<T> mNr = col_multiplier<T>(a, Kh, n1 / 2, kyr, n1, n2);
-                orr = cmul(scale(m0r + mNr, T(0.5)), zr) + cmul(scale(m0r - mNr, T(0.5)), conj(z));
+                o = packed_symbol(a, Kh, ky, n1, n2, z, zr);
+                orr = packed_symbol(a, Kh, kyr, n1, n2, zr, z);
                 if (ky == 0 && a.mode == COL_K) o.x = T(s_sigma);  // macroscopic stress
             }
             col[swz(ky)] = o;
@@ -1149,6 +1115,8 @@ template <typename T>
 cudaError_t configure_kernels(int n1, int n2) {
     if constexpr (std::is_same<T, double>::value) {
         return fix_configure(n1, n2);
+    } else if constexpr (std::is_same<T, float>::value) {
+        return f32_configure(n1, n2);
     } else {
         // the FFT kernels live on shared memory: allow large dynamic allocations and ask for the
         // largest shared-memory carveout so that several blocks stay resident per SM
@@ -1169,6 +1137,8 @@ void launch_row_forward(const Dev& d, const T* src0, const T* src1, cpx<T>* spec
                         int count, cudaStream_t s) {
     if constexpr (std::is_same<T, double>::value) {
         fix_row_forward(d, src0, src1, spec, partials, ctl, count, s);
+    } else if constexpr (std::is_same<T, float>::value) {
+        f32_row_forward(d, src0, src1, spec, partials, ctl, count, s);
     } else {
         const LaunchGeom& g = d.geom;
         dim3 grid(g.row_blocks, count);
@@ -1199,6 +1169,8 @@ void launch_col(const Dev& d, const cpx<T>* in, cpx<T>* out, int mode, bool with
                 int sym_odd2 = 0, int sym_imag = 0) {
     if constexpr (std::is_same<T, double>::value) {
         fix_col(d, in, out, col_args<T>(d, mode, with_mean, sym_odd2, sym_imag), count, s);
+    } else if constexpr (std::is_same<T, float>::value) {
+        f32_col(d, in, out, col_args<T>(d, mode, with_mean, sym_odd2, sym_imag), count, s);
     } else {
         const LaunchGeom& g = d.geom;
         dim3 grid(g.col_blocks, count);
@@ -1229,6 +1201,8 @@ void launch_row_inverse(const Dev& d, const cpx<T>* spec, T* dst, int mode, doub
                         cudaStream_t s, bool after_k = false) {
     if constexpr (std::is_same<T, double>::value) {
         fix_row_inverse(d, spec, dst, row_args<T>(d, mode, offset, after_k), count, s);
+    } else if constexpr (std::is_same<T, float>::value) {
+        f32_row_inverse(d, spec, dst, row_args<T>(d, mode, offset), count, s);
     } else {
         const LaunchGeom& g = d.geom;
         dim3 grid(g.row_blocks, count);

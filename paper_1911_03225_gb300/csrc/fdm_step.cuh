@@ -134,6 +134,49 @@ __device__ __forceinline__ cpx<T> col_apply(const ColArgs<T>& a, const T* __rest
     return mk(-(m.y * z.y), m.y * z.x);
 }
 
+// COL_K, by all threads of the block that holds the column kx = 0: <U13> from the row sums, then
+// the loading state of this step; *s_sigma is set by thread 0 (a barrier must follow)
+template <typename T>
+__device__ __forceinline__ void loading_from_rows(const ColArgs<T>& a, int n1, int n2, int inst, double* s_red,
+                                                  double* s_sigma) {
+    fdm_dev_scalars* sci = a.sc + inst;
+    const double* parts = a.row_partials ? a.row_partials + (size_t)inst * a.nparts : nullptr;
+    // <U13> from the row sums, then the loading state of this step (Sec. 5.1).  The
+    // order is fixed by n2 alone: kRedLanes compensated lane sums over a stride, then a
+    // fixed tree (results do not depend on the launch shape)
+    for (int v = threadIdx.x; v < kRedLanes; v += blockDim.x) {
+        double s = 0.0, c = 0.0;
+        for (int i = v; parts && i < a.nparts; i += kRedLanes) neumaier_add(s, c, parts[i]);
+        s_red[v] = s + c;
+    }
+    __syncthreads();
+    double tot = 0.0;
+    if (threadIdx.x < 32) {
+        double s = 0.0, c = 0.0;
+        for (int v = threadIdx.x; v < kRedLanes; v += 32) neumaier_add(s, c, s_red[v]);
+        tot = warp_sum(s + c);
+    }
+    if (threadIdx.x == 0) {
+        double mean = parts ? sci->phi_ref + tot / ((double)n1 * (double)n2) : sci->mean_up13;
+        double eps, sig;
+        loading_state(a.p, sci->step, sci->t, mean, &eps, &sig);
+        sci->mean_up13 = mean;
+        sci->eps_bar13 = eps;
+        sci->sigma_bar13 = sig;
+        *s_sigma = sig;
+    }
+}
+// the symbol on the packed column, z = C0 + i CN (C0, CN transforms of the real columns kx = 0 and
+// kx = n1/2): each multiplied by its own symbol and repacked,
+// out(ky) = (m0 + mN)/2 z(ky) + (m0 - mN)/2 conj(z(-ky))
+template <typename T>
+__device__ __forceinline__ cpx<T> packed_symbol(const ColArgs<T>& a, const T* __restrict__ Kh, int ky, int n1, int n2,
+                                                cpx<T> z, cpx<T> zr) {
+    cpx<T> m0 = col_multiplier<T>(a, Kh, 0, ky, n1, n2);
+    cpx<T> mN = col_multiplier<T>(a, Kh, n1 / 2, ky, n1, n2);
+    return cmul(scale(m0 + mN, T(0.5)), z) + cmul(scale(m0 - mN, T(0.5)), conj(zr));
+}
+
 enum RowMode { ROW_PLAIN = 0, ROW_TAU = 1 };
 
 // celerity law (Sec. 3.2.3 Hamiltonian; Sec. 4.1 prescribed), parameters in the field type
@@ -225,6 +268,13 @@ void fix_row_forward(const Dev& d, const double* src0, const double* src1, cpx<d
 void fix_col(const Dev& d, const cpx<double>* in, cpx<double>* out, const ColArgs<double>& a, int count,
              cudaStream_t s);
 void fix_row_inverse(const Dev& d, const cpx<double>* spec, double* dst, const RowArgs<double>& a, int count,
+                     cudaStream_t s);
+// the mixed path's transforms (fdm_f32.cu): the same for float fields
+cudaError_t f32_configure(int n1, int n2);
+void f32_row_forward(const Dev& d, const float* src0, const float* src1, cpx<float>* spec, double* partials,
+                     InstCtl ctl, int count, cudaStream_t s);
+void f32_col(const Dev& d, const cpx<float>* in, cpx<float>* out, const ColArgs<float>& a, int count, cudaStream_t s);
+void f32_row_inverse(const Dev& d, const cpx<float>* spec, float* dst, const RowArgs<float>& a, int count,
                      cudaStream_t s);
 void fix_tables(void* tw, int n, void* pt, int L, cudaStream_t s);
 
