@@ -441,7 +441,9 @@ __global__ void __launch_bounds__(FixBlock<L, true>::most, FixBlock<L, true>::mi
     const double phi_ref = (sci && a.vel.friction) ? sci->phi_ref : 0.0;
     // without friction and mobility factors |v0| = |M tau| (rounded once, monotone in |tau|), or
     // the prescribed |v0|: the largest |tau| is enough
-    const bool law = a.vel.friction || a.vel.mfac;
+    const bool law = a.mode == ROW_TAU && (a.vel.friction || a.vel.mfac);
+    VelLaw<double> plain = a.vel;
+    plain.friction = 0;
     for (int r0 = 0; r0 < R; r0 += RB) {
         const int y0 = blockIdx.x * R + r0;
         // pairs (k, L - k), k = lk + i T < L / 2, of row lr; k = 0 takes the middle L / 2.  After
@@ -506,24 +508,33 @@ __global__ void __launch_bounds__(FixBlock<L, true>::most, FixBlock<L, true>::mi
             for (int u = 0; u < 8; ++u) {
                 const size_t o = (size_t)(y0 + row) * (2 * L) + 2 * (j + u * T);
                 cpx<double> t = x[u];
-                if (a.mode == ROW_TAU) {
+                if (a.mode != ROW_TAU) {
+                    t = mk(t.x + a.offset, t.y + a.offset);
+                } else if (!a.vel.friction) {
                     double c0 = t.x, c1 = t.y;
-                    if (law) {
-                        cpx<double> w = mk(0.0, 0.0);
-                        if (a.vel.friction) w = *reinterpret_cast<const cpx<double>*>(up + o);
-                        c0 = celerity(a.vel, t.x, w.x, phi_ref);
-                        c1 = celerity(a.vel, t.y, w.y, phi_ref);
-                        if (a.vel.mfac) {
-                            const cpx<double> mf = *reinterpret_cast<const cpx<double>*>(a.vel.mfac + inst * nn + o);
-                            c0 = c0 * mf.x;
-                            c1 = c1 * mf.y;
-                        }
+                    if (a.vel.mfac) {
+                        const cpx<double> mf = *reinterpret_cast<const cpx<double>*>(a.vel.mfac + inst * nn + o);
+                        c0 = celerity(plain, t.x, 0.0, 0.0) * mf.x;
+                        c1 = celerity(plain, t.y, 0.0, 0.0) * mf.y;
                     }
                     vbits = max(vbits, max(ubits(c0) & kMagBits, ubits(c1) & kMagBits));
-                } else {
-                    t = mk(t.x + a.offset, t.y + a.offset);
                 }
                 *reinterpret_cast<cpx<double>*>(dst + o) = t;
+            }
+            if (a.mode == ROW_TAU && a.vel.friction) {   // from what was stored, one body for all values
+#pragma unroll 1
+                for (int u = 0; u < 8; ++u) {
+                    const size_t o = (size_t)(y0 + row) * (2 * L) + 2 * (j + u * T);
+                    const cpx<double> t = *reinterpret_cast<const cpx<double>*>(dst + o);
+                    const cpx<double> w = *reinterpret_cast<const cpx<double>*>(up + o);
+                    double c0 = celerity(a.vel, t.x, w.x, phi_ref), c1 = celerity(a.vel, t.y, w.y, phi_ref);
+                    if (a.vel.mfac) {
+                        const cpx<double> mf = *reinterpret_cast<const cpx<double>*>(a.vel.mfac + inst * nn + o);
+                        c0 = c0 * mf.x;
+                        c1 = c1 * mf.y;
+                    }
+                    vbits = max(vbits, max(ubits(c0) & kMagBits, ubits(c1) & kMagBits));
+                }
             }
         }
         if (r0 + RB < R) __syncthreads();

@@ -11,6 +11,8 @@
 // nothing overflows.  Measured against long-double transforms the result is closer than an
 // FP64 transform's for every field the library meets (noise, smooth fields, fronts).
 #pragma once
+#include <cmath>
+
 #include "fdm_device.cuh"
 
 namespace fdm {
@@ -321,6 +323,71 @@ FIX_HD long long fix_mulhi2(long long a, long long b, long long c, long long d, 
     const long long t = fix_mad(ch, dh, fix_wide(ah, bh));
     const long long q = fix_mad(cl, dh, fix_mad(ch, dl, fix_mad(al, bh, fix_mad(ah, bl, (long long)(0x80000000u >> s)))));
     return fix_combine(t, q, s);
+}
+// ---- cos(x / beta) for the lattice friction.  x becomes a fraction of a turn first: x / (2 pi beta)
+// modulo 1 comes from the product with the factor's leading 100 bits (exact to the fraction's
+// last bit, where a rounded x / beta is off by 2^-53 of its value), and the rest is a polynomial in 64-bit fixed point.
+struct FixTurns {
+    unsigned long long m, l;   // 1 / (2 pi |beta|) = (m + l 2^-64) 2^(e + 958)
+    int e;                     // beyond every exponent: beta outside the range below, use cos()
+};
+inline FixTurns fix_turns(double beta) {
+    FixTurns t{0ull, 0ull, 1 << 20};
+    const double b = beta < 0.0 ? -beta : beta;
+    if (!(b > 1e-100 && b < 1e100)) return t;
+    // 2 pi b and its reciprocal to about 104 bits, as sums of two doubles
+    const double p1 = 6.283185307179586, p2 = 2.4492935982947064e-16;
+    const double h = b * p1, l = std::fma(b, p1, -h) + b * p2;
+    const double r = 1.0 / h, dr = (std::fma(-r, h, 1.0) - r * l) * r;
+    int k;
+    const double f = std::frexp(r, &k);
+    const double d = std::ldexp(dr, 64 - k), df = std::floor(d);
+    t.m = ((unsigned long long)std::ldexp(f, 53) << 11) + (unsigned long long)(long long)df;
+    t.l = (unsigned long long)std::ldexp(d - df, 32) << 32;
+    t.e = k - 1022;
+    return t;
+}
+// cos(x / beta) in units of 2^-62, within 2^-59; false beyond 2^10 turns (there cos() of the
+// rounded x / beta is further than 1e-12 off, and its own bits are kept), infinities and NaN
+FIX_HD bool fix_cos(double x, const FixTurns& t, long long* c) {
+    const unsigned long long u = fix_bits(x);
+    const int E = (int)(u >> 52) & 0x7ff, k = E + t.e;
+    if (k > 10) return false;
+    const unsigned long long m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
+#if defined(__CUDA_ARCH__)
+    const unsigned long long lo0 = m * t.m, lo = lo0 + __umul64hi(m, t.l);
+    const unsigned long long hi = __umul64hi(m, t.m) + (lo < lo0 ? 1u : 0u);
+    unsigned long long F;
+    if (k > 0) F = (hi << k) | (lo >> (64 - k));
+    else asm("shr.u64 %0, %1, %2;" : "=l"(F) : "l"(hi), "r"(-k));   // 0 beyond 63
+#else
+    const unsigned __int128 P = (unsigned __int128)m * t.m + (((unsigned __int128)m * t.l) >> 64);
+    const unsigned long long hi = (unsigned long long)(P >> 64), lo = (unsigned long long)P;
+    const unsigned long long F = k > 0 ? (hi << k) | (lo >> (64 - k)) : (-k > 63 ? 0ull : hi >> -k);
+#endif
+    // F: the turn's fraction in 2^-64; cos(2 pi F) = sin(pi h / 2), h = 1 - 4 |F| in quarter turns of 2^62
+    const long long s = (long long)F >> 63;
+    const long long h = (long long)(0x4000000000000000ull - ((F ^ (unsigned long long)s) - (unsigned long long)s));
+    long long z = fix_mulhi(h, h, 2);
+    z -= z >> 62;
+    // the Taylor series of sin(pi h / 2) / h in z = h^2, (-1)^n (pi / 2)^(2n + 1) / (2n + 1)!, in
+    // 2^-62, to n = 11 (the next is below 2^-67).  From n = 7 on 32 bits hold the terms, in 2^-60 and
+    // each scaled by 4 more, since z comes in 2^-30.
+    const int y = (int)(z >> 32);
+    int w = -370;
+    w = 18974 + fix_hi(fix_wide(w, y));
+    w = -807426 + fix_hi(fix_wide(w, y));
+    w = 27978803 + fix_hi(fix_wide(w, y));
+    w = -771077950 + fix_hi(fix_wide(w, y));
+    long long p = 262505142787ll + fix_mulhi((long long)w, z, 4);
+    p = -16596735030340ll + fix_mulhi(p, z, 2);
+    p = 739904368663792ll + fix_mulhi(p, z, 2);
+    p = -21590780087563799ll + fix_mulhi(p, z, 2);
+    p = 367517370231208053ll + fix_mulhi(p, z, 2);
+    p = -2978983596875621757ll + fix_mulhi(p, z, 2);
+    p = 7244019458077122842ll + fix_mulhi(p, z, 2);
+    *c = fix_mulhi(h, p, 2);
+    return true;
 }
 // of one sign and none zero: the one of least magnitude, else 0
 FIX_HD long long fix_minmod3(long long a, long long b, long long c) {

@@ -2,6 +2,7 @@
 // law, the column pass's symbols, the celerity law and the time-step rule.
 #pragma once
 #include "fdm_device.cuh"
+#include "fdm_fix.cuh"
 #include "fdm_internal.h"
 
 namespace fdm {
@@ -186,6 +187,7 @@ struct VelLaw {
     int friction;        // tau_y != 0 and stress driven
     T v0, mobility;
     double tau_y, beta;  // lattice friction (FP64; evaluated only when friction != 0)
+    FixTurns turns;      // beta for fix_cos (FP64 and double-word fields)
     const T* mfac;       // per-cell mobility factor m(x) (heterogeneous drag, Sec. 5.3), or null
 };
 
@@ -198,14 +200,27 @@ template <typename T> VelLaw<T> make_vel(const fdm_params& p, const void* mfac =
     v.mobility = T(p.mobility);
     v.tau_y = p.tau_y;
     v.beta = p.beta;
+    v.turns = fix_turns(p.beta);
     return v;
+}
+
+// cos(x / beta).  FP64 instructions are what a friction node costs (two lanes per SM): cos() and
+// the division are about 45 of them, fix_cos two and 170 integer ones.  512 x 256 in FP64: rows
+// inverse 34.9 us and stencil 42.2 with cos(), 27.8 and 28.1 with fix_cos (18 and 25 without
+// friction).  The mixed path keeps cos(): its long runs amplify any other rounding to 32 bits.
+template <typename T> __device__ __forceinline__ double friction_cos(const VelLaw<T>& v, double x) {
+    if constexpr (!std::is_same<T, float>::value) {
+        long long c;
+        if (fix_cos(x, v.turns, &c)) return fix_to(c, -62);
+    }
+    return cos(x / v.beta);
 }
 
 template <typename T>
 __device__ __forceinline__ T celerity(const VelLaw<T>& v, T tau, T up, double phi_ref) {
     if (v.mode == FDM_V_PRESCRIBED) return v.v0;
     if (!v.friction) return -(v.mobility * tau);
-    const T fr = T(v.tau_y * cos(((double)up + phi_ref) / v.beta));
+    const T fr = T(v.tau_y * friction_cos(v, (double)up + phi_ref));
     return v.mobility * (fr - tau);
 }
 
