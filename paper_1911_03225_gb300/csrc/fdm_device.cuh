@@ -509,8 +509,10 @@ template <typename T> __device__ __forceinline__ void speed_range(T h, T& ap, T&
 // along the axes included: of the coupled random field 99.7% of the nodes qualify at the start
 // and 98% after 150 steps.  An axis along which nothing varies (both derivatives, both limited
 // second differences and the cross differences zero) qualifies as well: its two weights of 1/2
-// belong to equal values.  knp_upwind_df2 (below) is this form for double words, fix_upwind
-// (fdm_fix.cuh) for FP64 fields.
+// belong to equal values.  fix_upwind (fdm_fix.cuh) is this form for FP64 fields.  (FP32: the same
+// skipping took as many instructions as it saved, 69.6 us either way.  Double words: 348 -> 209 us at
+// 2048^2, but a coupled run of 74 steps there amplified the weights' other rounding, 3e-14, to
+// 1e-8, so they keep the whole scheme.)
 // ---------------------------------------------------------------------------------
 
 // ---------------------------------------------------------------------------------
@@ -859,71 +861,6 @@ __device__ __forceinline__ df2 knp_node_df2(F f, df2 v0, df dt_h, df theta, int 
         acc = acc + nx[s] * accs;
     }
     return f0 + acc;   // the weights sum to one
-}
-
-// The short form for two nodes of double-word fields (knp_node_df2's conventions): oka and okb tell
-// whether the lanes qualify; fd(lane, i, j) is f(i, j) of one lane, for offsets that differ
-// between the lanes.  (FP32 fields keep knp_node_x2 for every node: its 32-bit reciprocal square
-// roots are cheap, and the same skipping took as many instructions as it saved, 69.6 us either way.)
-__device__ __forceinline__ bool one_sign(float a, float b) {
-    return (a > 0.0f && b > 0.0f) || (a < 0.0f && b < 0.0f);
-}
-__device__ __forceinline__ bool opposite(float v, float p) {
-    return ((__float_as_uint(v) ^ __float_as_uint(p)) >> 31) != 0;
-}
-__device__ __forceinline__ bool one_sign(df a, df b) { return one_sign(a.hi, b.hi); }
-template <typename F, typename FD>
-__device__ __forceinline__ df2 knp_upwind_df2(F f, FD fd, df2 v0, df dt_h, df theta, int theta_code, int time_level,
-                                              bool* oka, bool* okb) {
-    const df2 f0 = f(0, 0);
-    const df2 xm = f(-1, 0), xp = f(1, 0), ym = f(0, -1), yp = f(0, 1);
-    const df2 dxm3 = xm - f(-2, 0), dxm1 = f0 - xm, dxp1 = xp - f0, dxp3 = f(2, 0) - xp;
-    const df2 dym3 = ym - f(0, -2), dym1 = f0 - ym, dyp1 = yp - f0, dyp3 = f(0, 2) - yp;
-    const df2 cxl = theta_mul(dxp1 - dxm1, theta, theta_code), cyl = theta_mul(dyp1 - dym1, theta, theta_code);
-    const df2 Sxp = minmod3(theta_mul(dxp3 - dxp1, theta, theta_code), thalf(dxp3 - dxm1), cxl);
-    const df2 Sxm = minmod3(cxl, thalf(dxp1 - dxm3), theta_mul(dxm1 - dxm3, theta, theta_code));
-    const df2 Syp = minmod3(theta_mul(dyp3 - dyp1, theta, theta_code), thalf(dyp3 - dym1), cyl);
-    const df2 Sym = minmod3(cyl, thalf(dyp1 - dym3), theta_mul(dym1 - dym3, theta, theta_code));
-    const df2 px0 = dxp1 - thalf(Sxp), px1 = dxm1 + thalf(Sxm);
-    const df2 qy0 = dyp1 - thalf(Syp), qy1 = dym1 + thalf(Sym);
-    const bool sa = opposite(v0.hi.x, px0.hi.x), sb = opposite(v0.hi.y, px0.hi.y);
-    const bool ta = opposite(v0.hi.x, qy0.hi.x), tb = opposite(v0.hi.y, qy0.hi.y);
-    const df2 fx = sel2(sa, sb, dxp1, -dxm1), fy = sel2(ta, tb, yp, ym);
-    const df2 fc = mkdf2(fd(0, sa ? 1 : -1, ta ? 1 : -1), fd(1, sb ? 1 : -1, tb ? 1 : -1));
-    const df2 mixed = (fc - fy) - fx;
-    // yc: f(0, -cy), the x2 neighbour on the other side (a double word is zero where its high
-    // word is)
-    auto one_way = [&](int l, float p0, float p1, float q0, float q1, float Sx0, float Sx1, float Sy0, float Sy1,
-                       float mx, df fxl, df fyl, df yc, bool s, bool t) -> bool {
-        const bool x1 = one_sign(p0, p1), y1 = one_sign(q0, q1);
-        if (x1 && y1) return true;
-        if (!x1 && !(p0 == 0.0f && p1 == 0.0f)) return false;
-        if (!y1 && !(q0 == 0.0f && q1 == 0.0f)) return false;
-        if (!x1 && !y1) return true;   // no gradient: H = 0
-        if (x1) return Sy0 == 0.0f && Sy1 == 0.0f && mx == 0.0f && ((fd(l, s ? 1 : -1, t ? -1 : 1) - yc) - fxl).hi == 0.0f;
-        return Sx0 == 0.0f && Sx1 == 0.0f && mx == 0.0f && (fd(l, s ? -1 : 1, t ? 1 : -1) - fyl).hi == 0.0f;
-    };
-    *oka = one_way(0, px0.hi.x, px1.hi.x, qy0.hi.x, qy1.hi.x, Sxp.hi.x, Sxm.hi.x, Syp.hi.x, Sym.hi.x, mixed.hi.x,
-                   lane(fx, 0), lane(fy, 0), lane(ta ? ym : yp, 0), sa, ta);
-    *okb = one_way(1, px0.hi.y, px1.hi.y, qy0.hi.y, qy1.hi.y, Sxp.hi.y, Sxm.hi.y, Syp.hi.y, Sym.hi.y, mixed.hi.y,
-                   lane(fx, 1), lane(fy, 1), lane(tb ? ym : yp, 1), sb, tb);
-    const df2 cross = sel2(sa == ta, sb == tb, mixed, -mixed);
-    const df2 Sx = sel2(sa, sb, Sxp, Sxm), Sy = sel2(ta, tb, Syp, Sym);
-    df2 p = sel2(sa, sb, px0, px1), q = sel2(ta, tb, qy0, qy1);
-    const df2 zero = bcast2(df(0.0f));
-    const df2 vdt = v0 * bcast2(dt_h);
-    if (time_level == 0) {
-        const df2 r2 = p * p + q * q;
-        const bool g0 = tguard(lane(r2, 0)), g1 = tguard(lane(r2, 1));
-        const df2 w = thalf(vdt) * trsqrt(r2);
-        const df2 np = p - w * (Sx * p + cross * q);
-        const df2 nq = q - w * (cross * p + Sy * q);
-        p = sel2(g0, g1, np, p);
-        q = sel2(g0, g1, nq, q);
-    }
-    const df2 s2 = p * p + q * q;
-    const df2 g = sel2(tguard(lane(s2, 0)), tguard(lane(s2, 1)), s2 * trsqrt(s2), zero);
-    return f0 - vdt * g;
 }
 
 }  // namespace fdm

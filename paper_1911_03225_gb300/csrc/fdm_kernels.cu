@@ -374,22 +374,20 @@ template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed 
 };
 
 // grid (n1 / tx, n2 / (ty npt), instances); block (tx, ty); thread (i, j) updates the
-// nodes (bx + i, by + j + k ty), k < npt.  FP64 and double words: first the nodes that have one
-// characteristic direction (fix_upwind, knp_upwind_df2), nearly all of them on the fields the method meets; each
-// warp lists its others and works through them with the whole scheme (fix_node,
-// knp_node_df2), 32 (or 64) at a
-// time.  What is left over, seldom a full warp's worth, goes on the instance's list in global
+// nodes (bx + i, by + j + k ty), k < npt.  FP64: first the nodes that have one characteristic
+// direction (fix_upwind), nearly all of them on the fields the method meets; each warp lists its
+// others and works through them with the whole scheme (fix_node), 32 at a time.  What is left over, seldom a full warp's worth, goes on the instance's list in global
 // memory when the launch has several waves of blocks (the list lies in the spectrum's buffer,
 // free between the inverse row kernel and the next step's forward one): the warp that completes
-// a chunk of 32 (64) of the list works through it, and the instance's last block takes the rest.
+// a chunk of 32 of the list works through it, and the instance's last block takes the rest.
 // On a launch that the GPU holds at once there are idle lanes to spare, and a tail would cost a
-// scheme's latency: each warp sees to its own, and double words take the whole scheme throughout
-// (128^2: 16 us against 20 for one form after the other).  No barrier follows the tile's
+// scheme's latency: each warp sees to its own (128^2: 16 us against 20).  No barrier follows the tile's
 // loads, so warps at the whole scheme and warps at the short one share the pipes.  A node's
 // result depends on the node alone, not on the lists.  2048^2, random field after 30 steps: FP64
-// 1388 -> 221 us (624 with the short form in FP64 arithmetic), double words 348 -> 209 us (lists
-// per block, behind a barrier: 733 and 369; per warp only: 759 and 426).  What bounds the FP64
-// kernel now is instruction issue: 54% of the slots, the integer pipe 57% and the FP64 pipe 49%
+// 1388 -> 221 us (624 with the short form in FP64 arithmetic; lists per block, behind a barrier,
+// 733; per warp only 759).  Double words and FP32 take the whole scheme at every node: their long
+// coupled runs amplify any other rounding beyond what two such runs may differ by.  What bounds
+// the FP64 kernel now is instruction issue: 54% of the slots, the integer pipe 57% and the FP64 pipe 49%
 // busy.
 // body of one block: the tile (tbx, tby) of instance inst, ntiles tiles per instance (the
 // last to start advances the clock); thread (tx_, ty_) of a tx x TY block
@@ -511,8 +509,8 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 lo_out[(size_t)yb * n1 + x] = lo;
             }
         }
-    } else if constexpr (std::is_same<T, df>::value && !GATHER) {
-        // double words on a small launch: the whole scheme for every node, two at once in the
+    } else if constexpr (std::is_same<T, df>::value) {
+        // double words: the whole scheme for every node, two at once in the
         // lanes of the packed FP32 instructions, an odd last one paired with itself and written once
 #pragma unroll 1
         for (int k = 0; k < npt; k += 2) {
@@ -546,38 +544,17 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
             if (a.vel.mfac) c = c * a.vel.mfac[inst * nn + o];
             return c;
         };
-        constexpr bool kTwo = std::is_same<T, df>::value;   // two nodes at once
-        constexpr int kRound = kTwo ? 64 : 32;              // nodes a warp takes at a time
-        if constexpr (kTwo) {
-            // in the lanes of the packed FP32 instructions (double words), an odd last node paired
-            // with itself and written once
+        constexpr int kRound = 32;   // nodes a warp takes at a time
 #pragma unroll 1
-            for (int k = 0; k < npt; k += 2) {
-                const int k2 = (k + 1 < npt) ? k + 1 : k;
-                const int ra = ty_ + k * TY, rb = ty_ + k2 * TY, la = ra + 2, lb = rb + 2;
-                auto f = [&](int i, int j) -> df2 { return mkdf2(tile[la + j][lx + i], tile[lb + j][lx + i]); };
-                auto fd = [&](int l, int i, int j) -> df { return tile[(l == 0 ? la : lb) + j][lx + i]; };
-                const size_t oa = place(ra, tx_), ob = place(rb, tx_);
-                const df2 v0 = mkdf2(velocity(oa, s_tau[ra][tx_], tile[la][lx]), velocity(ob, s_tau[rb][tx_], tile[lb][lx]));
-                bool oka, okb;
-                const df2 res = knp_upwind_df2(f, fd, v0, dt, a.theta, a.theta_code, a.time_level, &oka, &okb);
-                if (oka) out[oa] = lane(res, 0);
-                if (okb && k2 != k) out[ob] = lane(res, 1);
-                defer(!oka, ra);
-                defer(!okb && k2 != k, rb);
-            }
-        } else {
-#pragma unroll 1
-            for (int k = 0; k < npt; ++k) {
-                const int r = ty_ + k * TY, ly = r + 2;
-                auto f = [&](int i, int j) -> T { return tile[ly + j][lx + i]; };
-                const size_t o = place(r, tx_);
-                T res;
-                const bool ok = fix_upwind(f, velocity(o, s_tau[r][tx_], tile[ly][lx]), dt, a.theta_fix, a.time_level,
-                                           &res);
-                if (ok) out[o] = res;
-                defer(!ok, r);
-            }
+        for (int k = 0; k < npt; ++k) {
+            const int r = ty_ + k * TY, ly = r + 2;
+            auto f = [&](int i, int j) -> T { return tile[ly + j][lx + i]; };
+            const size_t o = place(r, tx_);
+            T res;
+            const bool ok = fix_upwind(f, velocity(o, s_tau[r][tx_], tile[ly][lx]), dt, a.theta_fix, a.time_level,
+                                       &res);
+            if (ok) out[o] = res;
+            defer(!ok, r);
         }
         __syncwarp();
         const int ln = tid & 31;
@@ -659,45 +636,27 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
             };
             auto at = [&](int x, int y, int i, int j) -> T { return u[((y + j) & my) * pitch + ((x + i) & mx)]; };
             auto where = [&](int x, int y) -> size_t { return c < 0 ? place(y, x) : (size_t)y * n1 + x; };
-            if constexpr (kTwo) {
-                if (2 * ln < m) {
-                    int xa, ya, xb, yb;
-                    node(2 * ln, &xa, &ya);
-                    node(2 * ln + 1 < m ? 2 * ln + 1 : 2 * ln, &xb, &yb);
-                    const size_t oa = where(xa, ya), ob = where(xb, yb);
-                    auto f = [&](int i, int j) -> df2 { return mkdf2(at(xa, ya, i, j), at(xb, yb, i, j)); };
-                    const df2 v0 = mkdf2(velocity(oa, st[ya * tpitch + xa], at(xa, ya, 0, 0)),
-                                         velocity(ob, st[yb * tpitch + xb], at(xb, yb, 0, 0)));
-                    const df2 res = knp_node_df2(f, v0, dt, a.theta, a.theta_code, a.time_level);
-                    out[oa] = lane(res, 0);
-                    if (ob != oa) out[ob] = lane(res, 1);
-                }
-            } else {
-                if (ln < m) {
-                    int x, y;
-                    node(ln, &x, &y);
-                    const size_t o = where(x, y);
-                    auto f = [&](int i, int j) -> T { return at(x, y, i, j); };
-                    out[o] = fix_node(f, velocity(o, st[y * tpitch + x], f(0, 0)), dt, a.theta_fix, a.time_level);
-                }
+            if (ln < m) {
+                int x, y;
+                node(ln, &x, &y);
+                const size_t o = where(x, y);
+                auto f = [&](int i, int j) -> T { return at(x, y, i, j); };
+                out[o] = fix_node(f, velocity(o, st[y * tpitch + x], f(0, 0)), dt, a.theta_fix, a.time_level);
             }
             if (c < 0) done += m;
         }
     }
 }
 
-// Blocks per SM the kernel is compiled for: the shape's own figure in FP32; four of 256 threads (64
-// registers, some spilled) in FP64, whose forms wait on long integer chains (2048^2 random field:
-// 327 us with two, 272 with three, 241 with four, 238 with five); in double words four for the
-// tallest tiles, which large grids take (2048^2: 247, 215 and 209 us with two, three and four), and
-// the shape's figure for the others (512^2: 33 us with two, 46 with four)
-template <typename T, int V, bool GATHER> constexpr int knp_blocks() {
-    if (std::is_same<T, float>::value || KnpShapes<T>::ty[V] != 8) return KnpShapes<T>::minb[V];
-    return std::is_same<T, double>::value || (GATHER && KnpShapes<T>::npt[V] == 4) ? 4 : KnpShapes<T>::minb[V];
+// Blocks per SM the kernel is compiled for: the shape's own figure; in FP64 four of 256 threads (64
+// registers, some spilled), whose forms wait on long integer chains (2048^2 random field: 327 us
+// with two, 272 with three, 241 with four, 238 with five)
+template <typename T, int V> constexpr int knp_blocks() {
+    return std::is_same<T, double>::value && KnpShapes<T>::ty[V] == 8 ? 4 : KnpShapes<T>::minb[V];
 }
 
 template <typename T, int V, bool GATHER>
-__global__ void __launch_bounds__(TX * KnpShapes<T>::ty[V], knp_blocks<T, V, GATHER>())
+__global__ void __launch_bounds__(TX * KnpShapes<T>::ty[V], knp_blocks<T, V>())
     knp_step_kernel(const T* phi0, const T* phi1, const T* __restrict__ tau0, int n1, int n2, int npt,
                     KnpArgs<T> a) {
     knp_step_body<T, V, GATHER>(phi0, phi1, tau0, n1, n2, npt, a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x * gridDim.y,
@@ -1222,7 +1181,7 @@ void launch_knp_shape(const Dev& d, const KnpArgs<T>& a, cudaStream_t s) {
     // lists (knp_step_body) from the size at which a launch takes several waves of blocks, counted
     // at two blocks of 256 threads per SM
     const bool gather = (size_t)grid.x * grid.y * grid.z * tx * TY > (size_t)2 * 152 * 2 * 256;
-    if constexpr (!std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, double>::value) {
         if (gather) {
             knp_step_kernel<T, V, true><<<grid, block, 0, s>>>((const T*)d.phi[0], (const T*)d.phi[1], (const T*)d.tau,
                                                                d.p.n1, d.p.n2, npt, a);

@@ -187,7 +187,7 @@ struct VelLaw {
     int friction;        // tau_y != 0 and stress driven
     T v0, mobility;
     double tau_y, beta;  // lattice friction (FP64; evaluated only when friction != 0)
-    FixTurns turns;      // beta for fix_cos (FP64 and double-word fields)
+    FixTurns turns;      // beta for fix_cos (FP64 fields)
     const T* mfac;       // per-cell mobility factor m(x) (heterogeneous drag, Sec. 5.3), or null
 };
 
@@ -207,9 +207,9 @@ template <typename T> VelLaw<T> make_vel(const fdm_params& p, const void* mfac =
 // cos(x / beta).  FP64 instructions are what a friction node costs (two lanes per SM): cos() and
 // the division are about 45 of them, fix_cos two and 170 integer ones.  512 x 256 in FP64: rows
 // inverse 34.9 us and stencil 42.2 with cos(), 27.8 and 28.1 with fix_cos (18 and 25 without
-// friction).  The mixed path keeps cos(): its long runs amplify any other rounding to 32 bits.
+// friction).  The other paths keep cos(), whose roundings their long runs amplify.
 template <typename T> __device__ __forceinline__ double friction_cos(const VelLaw<T>& v, double x) {
-    if constexpr (!std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, double>::value) {
         long long c;
         if (fix_cos(x, v.turns, &c)) return fix_to(c, -62);
     }
