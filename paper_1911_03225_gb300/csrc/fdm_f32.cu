@@ -189,12 +189,6 @@ __global__ void __launch_bounds__(F32Block<L>::most, F32Block<L>::minb)
     __shared__ double s_red[kRedLanes];
     constexpr int T = L / 8, n2 = L;
     const int inst = blockIdx.y, tid = threadIdx.x;
-    if (tid == 0) {
-        InstCtl ctl{a.mode == COL_K ? a.sc : nullptr, a.gated};
-        inst_state(ctl, inst, &s_run, &s_cur);
-    }
-    __syncthreads();
-    if (!s_run) return;
     const size_t half_n = (size_t)n1 * n2 / 2;
     in += inst * half_n;
     out += inst * half_n;
@@ -203,13 +197,23 @@ __global__ void __launch_bounds__(F32Block<L>::most, F32Block<L>::minb)
     cf* B = A + f32_slots(L, CB) * ld;
     const int c = tid / T, j = tid & (T - 1);
     const bool on = c < CB;
+    cf v[8];
+    auto load = [&](int kx) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = on ? load_once(in + (size_t)kx * n2 + j + u * T) : mk(0.0f, 0.0f);
+    };
+    load(blockIdx.x * C + c);   // on its way while thread 0 reads the instance's state
+    if (tid == 0) {
+        InstCtl ctl{a.mode == COL_K ? a.sc : nullptr, a.gated};
+        inst_state(ctl, inst, &s_run, &s_cur);
+    }
+    __syncthreads();
+    if (!s_run) return;
     const bool symbol = a.mode != COL_FWD && a.mode != COL_INV;
     for (int c0 = 0; c0 < C; c0 += CB) {
         const int kx = blockIdx.x * C + c0 + c;
         const bool packed_block = symbol && blockIdx.x == 0 && c0 == 0;   // holds the column kx = 0
-        cf v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = on ? load_once(in + (size_t)kx * n2 + j + u * T) : mk(0.0f, 0.0f);
+        if (c0 > 0) load(kx);
         if (packed_block && a.mode == COL_K) loading_from_rows(a, n1, n2, inst, s_red, &s_sigma);
         cf* X = A + c * ld;
         cf* Y = B + c * ld;
@@ -266,12 +270,6 @@ __global__ void __launch_bounds__(F32Block<L>::most, F32Block<L>::minb)
     __shared__ int s_run, s_cur;
     constexpr int T = L / 8;
     const int inst = blockIdx.y, tid = threadIdx.x;
-    if (tid == 0) {
-        InstCtl ctl{a.mode == ROW_TAU ? a.sc : nullptr, a.gated};
-        inst_state(ctl, inst, &s_run, &s_cur);
-    }
-    __syncthreads();
-    if (!s_run) return;
     const size_t nn = (size_t)(2 * L) * n2;
     spec += inst * (nn / 2);
     dst += inst * nn;
@@ -282,6 +280,24 @@ __global__ void __launch_bounds__(F32Block<L>::most, F32Block<L>::minb)
     const int row = tid / T, j = tid & (T - 1);
     const bool on = row < RB;
     const int lr = tid & (RB - 1), lk = tid >> lRB;   // the thread's row and first pair while loading
+    // pairs (k, L - k), k = lk + i T < L / 2, of row lr; k = 0 takes the middle L / 2
+    cf x[8];
+    auto load = [&](int y0) {
+        const cf* col = spec + y0 + lr;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = lk + i * T;
+            x[2 * i] = on ? load_once(col + (size_t)k * n2) : mk(0.0f, 0.0f);
+            x[2 * i + 1] = on ? load_once(col + (size_t)(k == 0 ? L / 2 : L - k) * n2) : mk(0.0f, 0.0f);
+        }
+    };
+    load(blockIdx.x * R);   // on its way while thread 0 reads the instance's state
+    if (tid == 0) {
+        InstCtl ctl{a.mode == ROW_TAU ? a.sc : nullptr, a.gated};
+        inst_state(ctl, inst, &s_run, &s_cur);
+    }
+    __syncthreads();
+    if (!s_run) return;
     float vmax = 0.0f;
     bool bad = false;
     const float* up = s_cur ? (const float*)a.phi1 : (const float*)a.phi0;
@@ -292,15 +308,7 @@ __global__ void __launch_bounds__(F32Block<L>::most, F32Block<L>::minb)
     plain.friction = 0;
     for (int r0 = 0; r0 < R; r0 += RB) {
         const int y0 = blockIdx.x * R + r0;
-        // pairs (k, L - k), k = lk + i T < L / 2, of row lr; k = 0 takes the middle L / 2
-        cf x[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = lk + i * T;
-            const cf* col = spec + y0 + lr;
-            x[2 * i] = on ? load_once(col + (size_t)k * n2) : mk(0.0f, 0.0f);
-            x[2 * i + 1] = on ? load_once(col + (size_t)(k == 0 ? L / 2 : L - k) * n2) : mk(0.0f, 0.0f);
-        }
+        if (r0 > 0) load(y0);
         if (on) {
             cf* Z = A + lr * ld;
 #pragma unroll

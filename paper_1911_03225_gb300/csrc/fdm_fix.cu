@@ -275,8 +275,9 @@ __device__ __forceinline__ void loading_block(const ColArgs<double>& a, int n1, 
     const double* parts = a.row_partials ? a.row_partials + (size_t)inst * a.nparts : nullptr;
     double s = 0.0, e = 0.0;
     if (parts && tid < T) {
+        neumaier_start(s, e, parts[tid]);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) neumaier_add(s, e, parts[tid + u * T]);
+        for (int u = 1; u < 8; ++u) neumaier_add(s, e, parts[tid + u * T]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -298,7 +299,7 @@ __device__ __forceinline__ void loading_block(const ColArgs<double>& a, int n1, 
     fdm_dev_scalars* sci = a.sc + inst;
     const double mean = parts ? sci->phi_ref + (tot + err) * a.scl : sci->mean_up13;
     double eps, sig;
-    loading_state(a.p, sci->step, sci->t, mean, &eps, &sig);
+    loading_state(a.p, a.mu, a.frac, sci->step, sci->t, mean, &eps, &sig);
     sci->mean_up13 = mean;
     sci->eps_bar13 = eps;
     sci->sigma_bar13 = sig;

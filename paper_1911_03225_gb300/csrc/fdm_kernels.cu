@@ -32,9 +32,8 @@ __device__ __forceinline__ void copy_async_wait_all() {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// Thread and residency bounds of the FFT kernels.  The FP32 kernels are latency bound: a
-// block of at most 512 threads with three resident per SM caps them at 40 registers, which
-// keeps 48 warps per SM instead of 32 (no spills).
+// Thread and residency bounds of the FFT kernels; a block's rows or columns hold at most eight
+// values per thread of these (FP32: 512 threads, as the launch shapes offered there)
 template <typename T> struct FftBounds { static constexpr int threads = 1024, minb = 1; };
 template <> struct FftBounds<float> { static constexpr int threads = 512, minb = 3; };
 
@@ -271,16 +270,23 @@ __device__ __forceinline__ void row_inverse_body(const cpx<T>* spec, T* dst, int
     const T* up = reinterpret_cast<const T*>(s_cur ? a.phi1 : a.phi0);
     if (up) up += inst * nn;
     const double phi_ref = (sci && a.vel.friction) ? sci->phi_ref : 0.0;
-    const bool need_up = a.vel.friction != 0;
+    VelLaw<T> plain = a.vel;   // without friction: no FP64 cosine on the path
+    plain.friction = 0;
     for (int e = threadIdx.x; e < R * L; e += blockDim.x) {
         int r = e >> lL, m = e & (L - 1);
         cpx<T> v = z[r * ld + swz(m)];
         size_t o = (size_t)(y0 + r) * n1 + 2 * m;
         // the pair (o, o + 1) moves as one aligned vector (o is even)
         if (a.mode == ROW_TAU) {
-            cpx<T> u = mk(T(0), T(0));
-            if (need_up) u = *reinterpret_cast<const cpx<T>*>(up + o);
-            T c0 = celerity(a.vel, v.x, u.x, phi_ref), c1 = celerity(a.vel, v.y, u.y, phi_ref);
+            T c0, c1;
+            if (a.vel.friction) {
+                const cpx<T> u = *reinterpret_cast<const cpx<T>*>(up + o);
+                c0 = celerity(a.vel, v.x, u.x, phi_ref);
+                c1 = celerity(a.vel, v.y, u.y, phi_ref);
+            } else {
+                c0 = celerity(plain, v.x, T(0), 0.0);
+                c1 = celerity(plain, v.y, T(0), 0.0);
+            }
             if (a.vel.mfac) {
                 const cpx<T> mf = *reinterpret_cast<const cpx<T>*>(a.vel.mfac + inst * nn + o);
                 c0 = c0 * mf.x;
@@ -1116,7 +1122,10 @@ ColArgs<T> col_args(const Dev& d, int mode, bool with_mean, int sym_odd2 = 0, in
     a.nparts = d.p.n2;
     a.sc = d.sc;
     a.gated = d.gated;
-    a.scl = T(1.0 / ((double)d.p.n1 * (double)d.p.n2));
+    a.inv_n = 1.0 / ((double)d.p.n1 * (double)d.p.n2);
+    a.scl = T(a.inv_n);
+    a.mu = d.p.E / (2.0 * (1.0 + d.p.nu));
+    a.frac = (double)d.p.nh / (double)d.p.nz;
     a.xi1_unit = T(6.283185307179586476925286766559 / ((double)d.p.n1 * d.p.dx));
     a.xi2_unit = T(6.283185307179586476925286766559 / ((double)d.p.n2 * d.p.dx));
     a.sym_odd2 = sym_odd2;

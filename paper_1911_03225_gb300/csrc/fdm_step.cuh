@@ -30,10 +30,12 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
     return (unsigned long long)__double_as_longlong(fabs(v));
 }
 
-__device__ __forceinline__ void loading_state(const fdm_params& p, long long step, double t, double mean,
-                                              double* eps, double* sig) {
-    const double mu = p.E / (2.0 * (1.0 + p.nu));
-    const double frac = (double)p.nh / (double)p.nz;
+// mu = E / (2 (1 + nu)) and frac = nh / nz come from the host: a division is about 12 FP64
+// instructions in a chain, 64 cycles each, and the chain that ends here is what the step's column
+// pass waits for on a small grid (128^2, us per step, with the divisions here and now: double words
+// 45 and 42, mixed 23.6 and 22)
+__device__ __forceinline__ void loading_state(const fdm_params& p, double mu, double frac, long long step, double t,
+                                              double mean, double* eps, double* sig) {
     if (p.loading_mode == FDM_LOAD_STRESS) {
         *sig = p.sigma_bar13;
         *eps = (p.sigma_bar13 + mu * frac * mean) / (2.0 * mu);
@@ -74,6 +76,11 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
     c += ((ubits(s) & kMagBits) >= (ubits(x) & kMagBits)) ? (s - t) + x : (x - t) + s;
     s = t;
 }
+// the first step, 0 + x with compensation 0 (not 0 for an infinite x)
+__device__ __forceinline__ void neumaier_start(double& s, double& c, double x) {
+    s = x;
+    c = x - x;
+}
 
 // Multiplier modes (all include the 1/(n1 n2) normalisation):
 //   COL_K         tau-hat = K U-hat, DC = sigma_bar13 (block 0 computes <U13> and loading)
@@ -97,6 +104,8 @@ struct ColArgs {
     fdm_dev_scalars* sc;         // COL_K: scalars of instance 0 (block 0 writes mean/eps/sigma)
     int gated;                   // COL_K: honour the instances' step budgets
     T scl;                       // 1 / (n1 n2)
+    double inv_n;                // the same (a power of two: a product with it is the quotient)
+    double mu, frac;             // COL_K: shear modulus; the layer's share of the cell
     T xi1_unit, xi2_unit;        // 2 pi / (n dx): xi = k~ * unit
     int sym_odd2, sym_imag;      // COL_SYM: symbol odd in xi2; symbol imaginary
 };
@@ -147,20 +156,22 @@ __device__ __forceinline__ void loading_from_rows(const ColArgs<T>& a, int n1, i
     // fixed tree (results do not depend on the launch shape)
     for (int v = threadIdx.x; v < kRedLanes; v += blockDim.x) {
         double s = 0.0, c = 0.0;
-        for (int i = v; parts && i < a.nparts; i += kRedLanes) neumaier_add(s, c, parts[i]);
+        if (parts && v < a.nparts) neumaier_start(s, c, parts[v]);
+        for (int i = v + kRedLanes; parts && i < a.nparts; i += kRedLanes) neumaier_add(s, c, parts[i]);
         s_red[v] = s + c;
     }
     __syncthreads();
     double tot = 0.0;
     if (threadIdx.x < 32) {
         double s = 0.0, c = 0.0;
-        for (int v = threadIdx.x; v < kRedLanes; v += 32) neumaier_add(s, c, s_red[v]);
+        neumaier_start(s, c, s_red[threadIdx.x]);
+        for (int v = threadIdx.x + 32; v < kRedLanes; v += 32) neumaier_add(s, c, s_red[v]);
         tot = warp_sum(s + c);
     }
     if (threadIdx.x == 0) {
-        double mean = parts ? sci->phi_ref + tot / ((double)n1 * (double)n2) : sci->mean_up13;
+        double mean = parts ? sci->phi_ref + tot * a.inv_n : sci->mean_up13;
         double eps, sig;
-        loading_state(a.p, sci->step, sci->t, mean, &eps, &sig);
+        loading_state(a.p, a.mu, a.frac, sci->step, sci->t, mean, &eps, &sig);
         sci->mean_up13 = mean;
         sci->eps_bar13 = eps;
         sci->sigma_bar13 = sig;
