@@ -66,11 +66,14 @@ def bytes_per_cell(elt, pair=False):
 #   v0 dt and v0 dt / 2 2; the row and column quadratics of the two sides 20 + 20;
 #   four corners of 36 (mixed difference 3, value 5, gradient 4, midpoint predictor 15,
 #   |grad| 5, Psi and its weight 4) 144; projection 5.  Total 250, of which 11 reciprocal
-#   square roots and one reciprocal.
+#   square roots and one reciprocal.  The mixed path does all of them at every node; the FP64 and
+#   double-word paths take a shorter form where one characteristic direction leaves three quadrants
+#   without weight, FP64 in integers, so no flop count of theirs compares with a flop rate.
 KNP_FLOPS_PER_CELL = 250
 
 
-KERNEL_SOURCES = ["fdm_kernels.cu", "fdm_device.cuh", "fdm_df.cuh", "fdm_internal.h"]
+KERNEL_SOURCES = ["fdm_kernels.cu", "fdm_fix.cu", "fdm_f32.cu", "fdm_step.cuh", "fdm_fix.cuh", "fdm_device.cuh", "fdm_df.cuh",
+                  "fdm_internal.h"]
 
 
 def kernel_source_hash():
@@ -299,20 +302,17 @@ def run_ours(args, world, rank, local):
     value = cells * K * world / (r["total_ms"] / 1e3)
 
     def roofline(prec, rr):
-        """Roofline of the step's dominant kernel: the stencil against the measured multiply-add
-        rate of its arithmetic (it is bound by arithmetic, not by HBM), the transforms
-        against the HBM peak."""
+        """Roofline of the step's dominant kernel: the mixed path's stencil against the measured
+        multiply-add rate of its arithmetic (it is bound by arithmetic, not by HBM), everything
+        else against the HBM peak."""
         d = rr["dominant"]
         d_ms = rr["phase_ms"][d]
         hbm_gbs = rr["bpc"][d] * cells / (d_ms / 1e3) / 1e9
-        if d == "knp_step":
-            key = {"fp64": "fp64", "df64": "df64", "mixed": "fp32"}[prec]
-            rl = {"bound": "alu", "achieved": KNP_FLOPS_PER_CELL * cells / (d_ms / 1e3) / 1e9, "peak": peaks[key],
+        if d == "knp_step" and prec == "mixed":
+            rl = {"bound": "alu", "achieved": KNP_FLOPS_PER_CELL * cells / (d_ms / 1e3) / 1e9, "peak": peaks["fp32"],
                   "unit": "GFLOP/s", "flops_per_cell": KNP_FLOPS_PER_CELL,
-                  "peak_source": "measured in this run (of measured): %s multiply-add chains on every SM, "
-                                 "fdm_measure_arith_rate, SM clock %s MHz" % (
-                                     {"fp64": "FP64", "fp32": "FP32", "df64": "double-word"}[key],
-                                     peaks["clocks"].get("sm_mhz"))}
+                  "peak_source": "measured in this run (of measured): FP32 multiply-add chains on every SM, "
+                                 "fdm_measure_arith_rate, SM clock %s MHz" % peaks["clocks"].get("sm_mhz")}
         else:
             rl = {"bound": "hbm", "achieved": hbm_gbs, "peak": hbm_peak, "unit": "GB/s", "peak_source": peak_src}
         rl["frac"] = rl["achieved"] / rl["peak"]
@@ -334,8 +334,9 @@ def run_ours(args, world, rank, local):
         roof["fp64_hbm_target"] = {
             "target_frac": FP64_HBM_TARGET_FRAC, "achieved_frac": roof["hbm_frac_of_step"],
             "met": roof["hbm_frac_of_step"] >= FP64_HBM_TARGET_FRAC,
-            "why": "the FP64 step is bound by the FP64 pipe, not by HBM: its %d B per cell take %.0f us of HBM "
-                   "time at the peak, its stencil alone %.0f us of FP64 multiply-adds at the measured rate" % (
+            "why": "the FP64 step (transforms and scheme in 64-bit fixed point) is bound by integer issue, not by "
+                   "HBM: its %d B per cell take %.0f us of HBM time at the peak, its stencil in floating point "
+                   "would take %.0f us of FP64 multiply-adds at the measured rate" % (
                        sum(r["bpc"].values()), sum(r["bpc"].values()) * cells / hbm_peak / 1e3,
                        KNP_FLOPS_PER_CELL * cells / peaks["fp64"] / 1e3)}
 
