@@ -66,9 +66,9 @@ fdm_status build_group(Dev& d, Arena& A, const fdm_params& p, int count, int gat
     if ((st = A.alloc((void**)&d.red, (size_t)6 * d.red_blocks * sizeof(double)))) return st;
     if ((st = A.alloc_host((void**)&d.red_host, kInfoScalarBytes + (size_t)6 * d.red_blocks * sizeof(double))))
         return st;
-    // the scalars and, behind them, the counters of the stencil's lists
+    // the scalars and, behind them, the counters of the FP64 stencil's lists
     const size_t sc_bytes = (size_t)count * sizeof(fdm_dev_scalars);
-    const size_t chunk_bytes = std::is_same<T, float>::value ? 0 : (size_t)count * list_chunks(n) * sizeof(unsigned);
+    const size_t chunk_bytes = std::is_same<T, double>::value ? (size_t)count * list_chunks(n) * sizeof(unsigned) : 0;
     if ((st = A.alloc((void**)&d.sc, sc_bytes + chunk_bytes))) return st;
     if (chunk_bytes) d.chunks = (unsigned*)((char*)d.sc + sc_bytes);
     FDM_CK(cudaMemsetAsync(d.sc, 0, sc_bytes + chunk_bytes, s));
@@ -534,7 +534,7 @@ size_t fdm_device_bytes(const fdm_params* p) {
     size_t n = (size_t)p->n1 * p->n2, e = elt_size(p);
     size_t nk = (size_t)(p->n1 / 2 + 1) * (p->n2 / 2 + 1);
     const size_t lo = p->precision == FDM_MIXED ? 2 * n * sizeof(float) : 0;   // low words of the state
-    const size_t list = p->precision == FDM_MIXED ? 0 : list_chunks(n) * sizeof(unsigned);
+    const size_t list = p->precision == FDM_FP64 ? list_chunks(n) * sizeof(unsigned) : 0;
     return 5 * n * e + lo + list + nk * e + (size_t)(p->n1 + p->n2) * 4 * e + (size_t)p->n2 * sizeof(double) + 64 * 1024;
 }
 

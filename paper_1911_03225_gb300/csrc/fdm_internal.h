@@ -64,7 +64,7 @@ struct Dev {
     double* red_host;      // pinned host copy: the instance's scalars, then the partials
     int red_blocks;
     fdm_dev_scalars* sc;   // [count]
-    unsigned* chunks;      // [count][list_chunks(n)]: entries in each chunk of the stencil's list
+    unsigned* chunks;      // FP64, [count][list_chunks(n)]: entries in each chunk of the stencil's list
     double phi_ref_host;   // single instance: host copy of sc[0].phi_ref
 };
 

@@ -412,8 +412,9 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
     __shared__ T s_tau[TY * NPT][TX];
     __shared__ T s_dt;
     __shared__ int s_run, s_cur;
-    // per warp: the nodes that need the whole scheme, as row * TX + column
-    __shared__ unsigned short s_list[kPair ? 1 : TY][kPair ? 1 : NPT * TX];
+    // FP64, per warp: the nodes that need the whole scheme, as row * TX + column
+    constexpr bool kLists = std::is_same<T, double>::value;
+    __shared__ unsigned short s_list[kLists ? TY : 1][kLists ? NPT * TX : 1];
     __shared__ int s_ended;   // warps done with their part of the tile
     const int rows = TY * npt;
     const int bx = tbx * tx, by = tby * rows;

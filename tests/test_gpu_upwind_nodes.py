@@ -1,7 +1,7 @@
-"""The FP64 and double-word stencils update nodes of one characteristic direction by a short form
-and collect the others for the whole scheme: fields that send every node, none, few or whole
-tiles to either, on launches of one wave and of several (where left-over nodes go through the
-instance's list), against the oracle.
+"""The FP64 stencil updates nodes of one characteristic direction by a short form and collects the
+others for the whole scheme: fields that send every node, none, few or whole tiles to either, on
+launches of one wave and of several (where left-over nodes go through the instance's list),
+against the oracle; double words, which take the whole scheme at every node, on the same fields.
 
 Tolerance (relative L2 of the increment): 1e-11, the parity bar of both paths; the increments are
 of the field's own size.  Three steps where minmod contracts rounding; one where it cannot: with
