@@ -398,14 +398,21 @@ FIX_HD long long fix_minmod3(long long a, long long b, long long c) {
     m = mc < m ? mc : m;
     return (m ^ s) & ~(m >> 63);
 }
-// the limiter parameter: code 1 or 2 when it is exactly that, else 2^-2 theta as fix_split's halves
+// the limiter parameter theta in [1, 2]: code 1 or 2 when it is exactly that, else 2^-3 theta as
+// fix_split's halves (2^-2 theta comes to 2^31 in the high half just below theta = 2)
 struct FixTheta { int code, h, l; };
+inline FixTheta fix_theta_of(double theta) {
+    FixTheta t;
+    t.code = theta == 1.0 ? 1 : (theta == 2.0 ? 2 : 0);
+    fix_split(0.125 * theta, &t.h, &t.l);
+    return t;
+}
 FIX_HD long long fix_theta(long long a, FixTheta t) {
     if (t.code == 1) return a;
     if (t.code == 2) return a + a;
     int h, l;
     fix_halves(a, h, l);
-    return fix_combine(fix_wide(h, t.h), fix_mad(l, t.h, fix_mad(h, t.l, 0x20000000ll)), 2);
+    return fix_combine(fix_wide(h, t.h), fix_mad(l, t.h, fix_mad(h, t.l, 0x10000000ll)), 3);
 }
 FIX_HD int fix_clz(long long v) {   // v > 0
 #if defined(__CUDA_ARCH__)

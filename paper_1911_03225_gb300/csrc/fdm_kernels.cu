@@ -1210,8 +1210,7 @@ KnpArgs<T> knp_args(const Dev& d) {
     a.lo1 = (const T*)d.phi_lo[1];
     a.theta = T(d.p.theta);
     a.theta_code = d.p.theta == 1.0 ? 1 : (d.p.theta == 2.0 ? 2 : 0);
-    a.theta_fix.code = a.theta_code;
-    fix_split(0.25 * d.p.theta, &a.theta_fix.h, &a.theta_fix.l);
+    a.theta_fix = fix_theta_of(d.p.theta);
     a.time_level = d.p.time_level;
     a.sc = d.sc;
     a.gated = d.gated;
