@@ -224,8 +224,9 @@ __device__ void smem_fft_ip(cpx<T>* a, int L, int nseq, int ld, const cpx<T>* __
 // P_k = X_k (1 <= k < n/2), from / to the n/2-point complex FFT of z_m = x_2m + i x_2m+1.
 // Z, P: one padded sequence each (L = n/2 entries).  W^k = exp(-2 pi i k / n) = tw_n[k].
 // ---------------------------------------------------------------------------------
-// exact halves
+// exact halves (the FP64 ones on the integer pipe, defined below)
 __device__ __forceinline__ float thalf(float x);
+__device__ __forceinline__ double thalf(double x);
 template <typename T> __device__ __forceinline__ cpx<T> chalf(cpx<T> a) { return mk(thalf(a.x), thalf(a.y)); }
 
 template <typename T> struct cpair { cpx<T> a, b; };
@@ -296,14 +297,15 @@ __device__ __forceinline__ float trcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double trcp(double x);   // on the FP32 and integer pipes, below
 // x / 2 (exact)
 __device__ __forceinline__ float thalf(float x) { return 0.5f * x; }
+__device__ __forceinline__ double thalf(double x);
 // x > 0 (false for zero and NaN)
 template <typename T> __device__ __forceinline__ bool tpos(T x) { return x > T(0); }
 
 // ---------------------------------------------------------------------------------
-// Decisions on doubles made on their bit patterns.  GB300's FP64 pipe retires 2 lanes per SM
-// per clock against 64 for the integer pipe, and comparisons, min/max and sign tests occupy it
-// like an FMA.  With the sign bit cleared, the bits of a double order like its magnitude (NaN
-// above infinity).
+// Decisions on doubles, and their exact scalings by 2, made on their bit patterns.  GB300's FP64
+// pipe retires 2 lanes per SM per clock against 64 for the integer pipe, and comparisons,
+// min/max, sign tests and multiplications by 1/2 or 2 occupy it like an FMA.  With the sign bit
+// cleared, the bits of a double order like its magnitude (NaN above infinity).
 // ---------------------------------------------------------------------------------
 constexpr unsigned long long kMagBits = 0x7fffffffffffffffull, kInfBits = 0x7ff0000000000000ull;
 __device__ __forceinline__ unsigned long long ubits(double x) { return (unsigned long long)__double_as_longlong(x); }
@@ -313,9 +315,33 @@ __device__ __forceinline__ bool tpos(double x) { return mag_ok(ubits(x)); }   //
 
 __device__ __forceinline__ double dbits(unsigned long long v) { return __longlong_as_double((long long)v); }
 
-// 1/sqrt(x) of a double x > 0 with no FP64 instruction (the Nye sums and the velocity readout
-// take square roots of doubles; GB300's FP64 pipe is 30 times slower than the pipes this runs
-// on).  Newton-Raphson iteration for x^(-1/2)
+// x / 2 exactly, on the integer pipe: one less in the exponent field for normal x above the
+// least normal exponent; zero, subnormals and the least normal exponent halve their
+// magnitude bits (ties to even, as the rounded product); infinities and NaN unchanged
+__device__ __forceinline__ double thalf(double x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+    if (__builtin_expect(e - 2u < 0x7fdu, 1)) return __hiloint2double(hi - 0x100000, lo);
+    if (e == 0x7ffu) return x;
+    const unsigned long long u = ubits(x), m = u & kMagBits;
+    return __longlong_as_double((long long)((u & ~kMagBits) | ((m >> 1) + (m & (m >> 1) & 1ull))));
+}
+// 2 x exactly, on the integer pipe: one more in the exponent field for normal x below the
+// largest exponent; zero and subnormals double their magnitude bits (exact, and carries
+// into the exponent field where the result is normal); the largest exponent (overflow to
+// infinity), infinities and NaN through the rounded sum
+__device__ __forceinline__ double ttwice(double x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+    if (__builtin_expect(e - 1u < 0x7fdu, 1)) return __hiloint2double(hi + 0x100000, lo);
+    if (e != 0u) return x + x;
+    const unsigned long long u = ubits(x);
+    return __longlong_as_double((long long)((u & ~kMagBits) | ((u & kMagBits) << 1)));
+}
+
+// 1/sqrt(x) of a double x > 0 with no FP64 instruction (the whole scheme at an FP64 node, knp_node,
+// and the Nye sums; GB300's FP64 pipe is 30 times slower than the pipes this runs on).
+// Newton-Raphson iteration for x^(-1/2)
 // (y <- y + y (1 - x y^2) / 2) from the single-precision special-function seed, with the
 // residuals formed from exact products (FMA TwoProd) and compensated sums (TwoSum) of FP32
 // numbers (the error-free transformations of Dekker and Knuth), every operation an explicitly
@@ -468,7 +494,8 @@ __device__ __forceinline__ double trcp(double x) {
 
 // ---------------------------------------------------------------------------------
 // Kurganov-Noelle-Petrova update of one node (Sec. 3.2.3 Steps 1-4; readings G1-G7): knp_node_x2
-// (two FP32 nodes), knp_node_df2 (two double-word nodes) and fix_node (FP64, fdm_fix.cuh).
+// (two FP32 nodes), knp_node_df2 (two double-word nodes) and knp_node (one FP64 node; most take
+// the short form fix_upwind, fdm_fix.cuh, instead).
 // f(i, j): value at node offset (i along x1, j along x2), i, j in [-2, 2].
 // ---------------------------------------------------------------------------------
 template <typename T> __device__ __forceinline__ T minmod3(T a, T b, T c) {
@@ -485,18 +512,146 @@ __device__ __forceinline__ bool tguard(double x) { return tpos(x); }
 // sqrt(x) for x >= 0
 template <typename T> __device__ __forceinline__ T tsqrt(T x) { return tguard(x) ? x * trsqrt(x) : T(0); }
 
-// |a| < |b|
+// the same function on bit patterns: when a, b, c are nonzero, not NaN and of one sign, the
+// one of least magnitude; else 0
+__device__ __forceinline__ double minmod3(double a, double b, double c) {
+    const unsigned long long ua = ubits(a), ub = ubits(b), uc = ubits(c);
+    const unsigned long long ma = ua & kMagBits, mb = ub & kMagBits, mc = uc & kMagBits;
+    const bool ok = ((((ua ^ ub) | (ua ^ uc)) >> 63) == 0) && mag_ok(ma) && mag_ok(mb) && mag_ok(mc);
+    double r = (mb < ma) ? b : a;
+    const unsigned long long mr = (mb < ma) ? mb : ma;
+    r = (mc < mr) ? c : r;
+    return ok ? r : 0.0;
+}
+
+// |a| < |b| (on bit patterns for FP64)
 __device__ __forceinline__ bool tmag_less(df a, df b) { return tabs(a) < tabs(b); }
+__device__ __forceinline__ bool tmag_less(double a, double b) { return (ubits(a) & kMagBits) < (ubits(b) & kMagBits); }
 
 // one-sided speeds: ap = max(ap, h), am = min(am, h) for ap >= 0 >= am, NaN ignored
 template <typename T> __device__ __forceinline__ void speed_range(T h, T& ap, T& am) {
     ap = tmax(ap, h);
     am = tmin(am, h);
 }
+__device__ __forceinline__ void speed_range(double h, double& ap, double& am) {
+    const unsigned long long u = ubits(h), m = u & kMagBits;
+    if (mag_ok(m)) {
+        if ((u >> 63) == 0) { if (m > ubits(ap)) ap = h; }
+        else if (m > (ubits(am) & kMagBits)) am = h;
+    }
+}
+
 // The update in cell units: with h the cell size, gradients are carried as h * grad (the
 // first differences themselves), displacements as d / h, and the time step as dt / h.  The
 // one-sided speeds depend only on the gradient's direction, so they are unchanged; every
 // formula of Steps 1-4 then holds with h = 1 and dt replaced by dt / h.
+// One FP64 node.  The products by theta are skipped or exact where they can be, the weights
+// w(s,t) = nx[s] ny[t] / (dxw dyw) take one reciprocal.
+template <typename F>
+__device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double theta, int theta_code, int time_level) {
+    using T = double;
+    auto theta_mul = [&](T x) -> T { return theta_code == 1 ? x : (theta_code == 2 ? ttwice(x) : theta * x); };
+    struct Side {  // one-dimensional limited quadratic on the cell on one side of the node
+        T D;  // first difference toward that side, signed as phi_{j+1}-phi_j or phi_j-phi_{j-1}
+        T S;  // limited second difference on that cell
+    };
+    const T f0 = f(0, 0);
+    // Step 1: first differences and limited second differences along x1 and x2
+    T dxm3 = f(-1, 0) - f(-2, 0), dxm1 = f0 - f(-1, 0), dxp1 = f(1, 0) - f0, dxp3 = f(2, 0) - f(1, 0);
+    T dym3 = f(0, -1) - f(0, -2), dym1 = f0 - f(0, -1), dyp1 = f(0, 1) - f0, dyp3 = f(0, 2) - f(0, 1);
+    Side xs[2], ys[2];  // [0] = + side, [1] = - side
+    {
+        const T c = theta_mul(dxp1 - dxm1);  // shared by both limiters
+        xs[0].D = dxp1; xs[0].S = minmod3(theta_mul(dxp3 - dxp1), thalf(dxp3 - dxm1), c);
+        xs[1].D = dxm1; xs[1].S = minmod3(c, thalf(dxp1 - dxm3), theta_mul(dxm1 - dxm3));
+    }
+    {
+        const T c = theta_mul(dyp1 - dym1);
+        ys[0].D = dyp1; ys[0].S = minmod3(theta_mul(dyp3 - dyp1), thalf(dyp3 - dym1), c);
+        ys[1].D = dym1; ys[1].S = minmod3(c, thalf(dyp1 - dym3), theta_mul(dym1 - dym3));
+    }
+    // one-sided derivatives at the node (times h)
+    T px[2] = {xs[0].D - thalf(xs[0].S), xs[1].D + thalf(xs[1].S)};
+    T qy[2] = {ys[0].D - thalf(ys[0].S), ys[1].D + thalf(ys[1].S)};
+    // Step 2: one-sided speeds over the four pairs (G4; dH/dp = v0 p / |(p,q)|, 0 at the
+    // origin).  For a fixed p the magnitude |p| / |(p,q)| falls as |q| grows and keeps its
+    // sign, so max(0, .) and min(0, .) of dH/dp over the pairs are attained with the q of
+    // least magnitude, and those of dH/dq with the p of least magnitude: the pairs
+    // (p0, qm), (p1, qm), (pm, qm'), where qm' is the other q, cover all four.
+    const bool tq = tmag_less(qy[1], qy[0]), tp = tmag_less(px[1], px[0]);
+    const T qm = tq ? qy[1] : qy[0], qo = tq ? qy[0] : qy[1];
+    const T pm = tp ? px[1] : px[0];
+    auto inv_norm = [&](T p, T q) -> T {   // v0 / |(p, q)|, 0 at the origin
+        const T r2 = p * p + q * q;
+        return tguard(r2) ? v0 * trsqrt(r2) : T(0);
+    };
+    const T r0 = inv_norm(px[0], qm), r1 = inv_norm(px[1], qm), rc = inv_norm(pm, qo);
+    T ap = T(0), am = T(0), bp = T(0), bm = T(0);
+    speed_range(r0 * px[0], ap, am);
+    speed_range(r1 * px[1], ap, am);
+    speed_range((tp ? r1 : r0) * qm, bp, bm);   // the pair (pm, qm) is (p0, qm) or (p1, qm)
+    speed_range(rc * qo, bp, bm);
+    // Step 4 weights (G1, G5): w(s,t) = nx[s] ny[t] / (dxw dyw), one reciprocal
+    T nx[2], ny[2], dxw = ap - am, dyw = bp - bm;
+    if (tguard(dxw)) { nx[0] = -am; nx[1] = ap; }
+    else { nx[0] = T(0.5); nx[1] = T(0.5); dxw = T(1); }
+    if (tguard(dyw)) { ny[0] = -bm; ny[1] = bp; }
+    else { ny[0] = T(0.5); ny[1] = T(0.5); dyw = T(1); }
+    const T inv_w = trcp(dxw * dyw);
+    const T vdt = v0 * dt_h;                 // v0 dt / h
+    const T hvdt = thalf(vdt);               // v0 dt / (2 h)
+    // Step 3: values at the four intermediate points (G2, G3).  Along each direction the
+    // limited quadratic on the side's cell, in cell units: with e the displacement / h and
+    // sg = -1 on the + side, +1 on the - side,  X(e) = D e + S e (e + sg) / 2 and
+    // h X'(e) = D + S (e + sg / 2).
+    T Y[2], dY[2], ey[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        ey[t] = (t == 0 ? bp : bm) * dt_h;
+        const T sgn = (t == 0) ? T(-1) : T(1);
+        Y[t] = ey[t] * (ys[t].D + thalf(ys[t].S) * (ey[t] + sgn));
+        dY[t] = ys[t].D + ys[t].S * (ey[t] + thalf(sgn));
+    }
+    T acc = T(0);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const int cx = (s == 0) ? 1 : -1;
+        const T ex = (s == 0 ? ap : am) * dt_h;
+        const T Dx = xs[s].D, Sx = xs[s].S;
+        const T sgn = (s == 0) ? T(-1) : T(1);
+        const T X = ex * (Dx + thalf(Sx) * (ex + sgn));
+        const T dX = Dx + Sx * (ex + thalf(sgn));
+        const T fx0 = (s == 0) ? Dx : -Dx;   // f(cx, 0) - f0, the side's first difference
+        T accs = T(0);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int cy = (t == 0) ? 1 : -1;
+            // mixed second difference of the quadrant cell (h^2 times the bilinear cross term)
+            const T mixed = (f(cx, cy) - f(0, cy)) - fx0;
+            const T cross = (cx * cy > 0) ? mixed : -mixed;
+            const T val = X + Y[t] + cross * ex * ey[t];   // minus f0, added once below
+            T p = dX + cross * ey[t];
+            T q = dY[t] + cross * ex;
+            if (time_level == 0) {
+                // (p, q) -= dt/2 Hess grad_(p,q) H, grad H = v0 (p, q) / |(p, q)|
+                const T r2 = p * p + q * q;
+                if (tguard(r2)) {
+                    const T w = hvdt * trsqrt(r2);
+                    const T np = p - w * (Sx * p + cross * q);
+                    const T nq = q - w * (cross * p + ys[t].S * q);
+                    p = np; q = nq;
+                }
+            }
+            const T s2 = p * p + q * q;
+            const T g = tguard(s2) ? s2 * trsqrt(s2) : T(0);   // h |grad|
+            const T psi = val - vdt * g;
+            accs += ny[t] * psi;
+        }
+        acc += nx[s] * accs;
+    }
+    return f0 + acc * inv_w;   // the weights sum to one
+}
+
 // ---------------------------------------------------------------------------------
 // Nodes of one characteristic direction.  Where both one-sided derivatives along x1 have one
 // sign, and both along x2 have one sign, every pair gives dH/dp of one sign and dH/dq of one

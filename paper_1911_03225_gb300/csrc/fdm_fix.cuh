@@ -538,160 +538,4 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
     return true;
 }
 
-FIX_HD float fix_rcp_seed(float x) {   // 1 / x, relative error below 2^-21
-#if defined(__CUDA_ARCH__)
-    return __fdividef(1.0f, x);
-#else
-    return 1.0f / x * (1.0f - 0x1p-22f);
-#endif
-}
-// a / w in units of 2^-61, 0 <= a <= w, 0 < w <= 2^62 (2^-58 absolute): the reciprocal of w scaled
-// to [1/2, 1) from the float seed y0 as y0 (1 + e + e^2), e = 1 - w y0 (the geometric series)
-FIX_HD long long fix_ratio(long long a, long long w) {
-    const int L = fix_clz(w) - 1;
-    const long long wn = (long long)((unsigned long long)w << L) >> 2, an = (long long)((unsigned long long)a << L) >> 2;
-    const float s = fix_rcp_seed((float)(unsigned)((unsigned long long)wn >> 29) * 0x1p-32f);
-    const int y = fix_round(s * 0x1p29f);
-    const long long one = (long long)1 << 58;
-    const long long e = one - fix_mulhi(wn, (long long)y << 32);   // 2^58 e, wn = 2^61 w
-    int eh, el;
-    fix_halves(e, eh, el);
-    const float ef = (float)(int)(e >> 16) * 0x1p-42f;
-    const long long r = fix_mad(fix_round(s * ef * ef * 0x1p60f), 1,
-                                ((long long)y << 31) + (fix_wide(y, eh) << 5) + (fix_wide(y, el) >> 27));
-    return fix_mulhi(an, r, 4);
-}
-// |(p, q)| of integers in a node's units (0 for (0, 0))
-FIX_HD long long fix_norm(long long p, long long q) {
-    long long ps, qs, r2;
-    int L;
-    if (!fix_norm2(p, q, &ps, &qs, &L, &r2)) return 0;
-    const long long r = fix_mulhi(r2 << 3, fix_rsqrt(r2)) << 3;
-    return (r + ((1ll << L) >> 1)) >> L;
-}
-// (p, q) / |(p, q)| in units of 2^-61 ((0, 0) for (0, 0))
-FIX_HD void fix_direction(long long p, long long q, long long* c, long long* s) {
-    long long ps, qs, r2;
-    int L;
-    *c = *s = 0;
-    if (!fix_norm2(p, q, &ps, &qs, &L, &r2)) return;
-    const long long y = fix_rsqrt(r2);
-    *c = fix_mulhi(ps, y, 3);
-    *s = fix_mulhi(qs, y, 3);
-}
-
-// The whole scheme for one FP64 node (Sec. 3.2.3 Steps 1-4, readings G1-G7) in cell units and
-// fixed point: the units of fix_upwind with E over all twelve differences.  The update is homogeneous in
-// U13, so a node near the ends of FP64's range is updated at 2^+-600 times its values; one with a
-// NaN, an infinity or a displacement beyond two cells (no finite step has one) gets a NaN.
-template <typename F>
-FIX_HD double fix_node(F f, double v0, double dt_h, FixTheta th, int time_level) {
-    auto top = [](unsigned a, unsigned b) { return a > b ? a : b; };
-    double k = 1.0, back = 1.0;
-    double a[12];
-    int E;
-#pragma unroll 1
-    for (int pass = 0;; ++pass) {
-        auto g = [&](int i, int j) { return pass ? f(i, j) * k : f(i, j); };
-        const double f0 = g(0, 0), xm = g(-1, 0), xp = g(1, 0), ym = g(0, -1), yp = g(0, 1);
-        a[0] = xm - g(-2, 0);
-        a[1] = f0 - xm;
-        a[2] = xp - f0;
-        a[3] = g(2, 0) - xp;
-        a[4] = ym - g(0, -2);
-        a[5] = f0 - ym;
-        a[6] = yp - f0;
-        a[7] = g(0, 2) - yp;
-        a[8] = g(1, 1) - yp;     // the quadrants' differences f(cx, cy) - f(0, cy)
-        a[9] = g(1, -1) - ym;
-        a[10] = g(-1, 1) - yp;
-        a[11] = g(-1, -1) - ym;
-        unsigned m = 0;
-#pragma unroll
-        for (int i = 0; i < 12; ++i) m = top(m, fix_mag(a[i]));
-        E = (int)(m >> 20);
-        if (pass || (E >= kFixLowExp && E <= kFixHighExp)) break;
-        const bool up = E < kFixLowExp;
-        k = up ? 0x1p600 : 0x1p-600;
-        back = up ? 0x1p-600 : 0x1p600;
-    }
-    const double vdt = v0 * dt_h;
-    if (E >= 0x7ff || (fix_mag(vdt) >> 20) > 1023u) return fix_from_bits(0x7ff8000000000000ull);
-    if (E < kFixLowExp) return f(0, 0);   // no difference, however scaled
-    const int Es = E;   // |differences| < 2^58
-    // Step 1
-    long long D[2][2], S[2][2], P[2][2];   // axis; side 0: +, 1: -
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        const long long m3 = fix_from<kFixBits, true>(a[4 * x], Es), m1 = fix_from<kFixBits, true>(a[4 * x + 1], Es), p1 = fix_from<kFixBits, true>(a[4 * x + 2], Es),
-                        p3 = fix_from<kFixBits, true>(a[4 * x + 3], Es);
-        const long long c = fix_theta(p1 - m1, th);
-        D[x][0] = p1;
-        D[x][1] = m1;
-        S[x][0] = fix_minmod3(fix_theta(p3 - p1, th), (p3 - m1) >> 1, c);
-        S[x][1] = fix_minmod3(c, (p1 - m3) >> 1, fix_theta(m1 - m3, th));
-        P[x][0] = p1 - (S[x][0] >> 1);
-        P[x][1] = m1 + (S[x][1] >> 1);
-    }
-    // Step 2: the one-sided displacements v0 dt dH/d(p, q) in units of 2^-61, from the three pairs
-    // that attain their extremes: |p| / |(p, q)| falls as |q| grows, so those of dH/dp belong to
-    // the q of least magnitude, those of dH/dq to the p of least magnitude
-    auto mag = [](long long v) { return v ^ (v >> 63); };
-    const bool tq = mag(P[1][1]) < mag(P[1][0]), tp = mag(P[0][1]) < mag(P[0][0]);
-    const long long qm = tq ? P[1][1] : P[1][0], qo = tq ? P[1][0] : P[1][1], pm = tp ? P[0][1] : P[0][0];
-    const long long h = fix_from<kFixBits, true>(vdt, 1023) << 4;   // v0 dt / h in units of 2^-61
-    long long c0, c1, cc, s0, s1, so;
-    fix_direction(P[0][0], qm, &c0, &s0);
-    fix_direction(P[0][1], qm, &c1, &s1);
-    fix_direction(pm, qo, &cc, &so);
-    const long long e[2][2] = {{fix_mulhi(c0, h, 3), fix_mulhi(c1, h, 3)}, {fix_mulhi(tp ? s1 : s0, h, 3), fix_mulhi(so, h, 3)}};
-    long long d[2][2], w[2][2];   // displacements and weights of each axis's sides
-    const long long one = (long long)1 << 61;
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        const long long hi = e[x][0] > e[x][1] ? e[x][0] : e[x][1], lo = e[x][0] < e[x][1] ? e[x][0] : e[x][1];
-        d[x][0] = hi > 0 ? hi : 0;
-        d[x][1] = lo < 0 ? lo : 0;
-        const long long span = d[x][0] - d[x][1];
-        w[x][1] = span > 0 ? fix_ratio(d[x][0], span) : one >> 1;
-        w[x][0] = one - w[x][1];
-    }
-    // Step 3: along each axis X(e) = e (D + S (e + sg) / 2) and its derivative D + S (e + sg / 2)
-    long long X[2][2], dX[2][2];
-#pragma unroll
-    for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const long long sg = s == 0 ? -one : one;
-            X[x][s] = fix_mulhi(D[x][s] + fix_mulhi(S[x][s] >> 1, d[x][s] + sg, 3), d[x][s], 3);
-            dX[x][s] = D[x][s] + fix_mulhi(S[x][s], d[x][s] + (sg >> 1), 3);
-        }
-    long long acc = 0;
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        if (w[0][s] == 0) continue;
-        long long accs = 0;
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-            if (w[1][t] == 0) continue;
-            const long long mixed = fix_from<kFixBits, true>(a[8 + 2 * s + t], Es) - (s == 0 ? D[0][0] : -D[0][1]);
-            const long long cross = (s == t) ? mixed : -mixed;
-            const long long cx = fix_mulhi(cross, d[0][s], 3);
-            const long long val = X[0][s] + X[1][t] + fix_mulhi(cx, d[1][t], 3);
-            long long p = dX[0][s] + fix_mulhi(cross, d[1][t], 3), q = dX[1][t] + cx;
-            if (time_level == 0) {
-                // (p, q) -= dt/2 Hess grad_(p,q) H, grad H = v0 (p, q) / |(p, q)|
-                long long c, n;
-                fix_direction(p, q, &c, &n);
-                p -= fix_mulhi(fix_mulhi2(S[0][s], c, cross, n, 3), h, 2);
-                q -= fix_mulhi(fix_mulhi2(cross, c, S[1][t], n, 3), h, 2);
-            }
-            const long long psi = val - fix_mulhi(fix_norm(p, q), h, 3);
-            accs += fix_mulhi(psi, w[1][t], 3);
-        }
-        acc += fix_mulhi(accs, w[0][s], 3);   // Step 4
-    }
-    return f(0, 0) + fix_to(acc, Es - 1080) * back;
-}
-
 }  // namespace fdm

@@ -382,19 +382,18 @@ template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed 
 // grid (n1 / tx, n2 / (ty npt), instances); block (tx, ty); thread (i, j) updates the
 // nodes (bx + i, by + j + k ty), k < npt.  FP64: first the nodes that have one characteristic
 // direction (fix_upwind), nearly all of them on the fields the method meets; each warp lists its
-// others and works through them with the whole scheme (fix_node), 32 at a time.  What is left over, seldom a full warp's worth, goes on the instance's list in global
-// memory when the launch has several waves of blocks (the list lies in the spectrum's buffer,
-// free between the inverse row kernel and the next step's forward one): the warp that completes
-// a chunk of 32 of the list works through it, and the instance's last block takes the rest.
-// On a launch that the GPU holds at once there are idle lanes to spare, and a tail would cost a
-// scheme's latency: each warp sees to its own (128^2: 16 us against 20).  No barrier follows the tile's
-// loads, so warps at the whole scheme and warps at the short one share the pipes.  A node's
-// result depends on the node alone, not on the lists.  2048^2, random field after 30 steps: FP64
-// 1388 -> 221 us (624 with the short form in FP64 arithmetic; lists per block, behind a barrier,
-// 733; per warp only 759).  Double words and FP32 take the whole scheme at every node: their long
-// coupled runs amplify any other rounding beyond what two such runs may differ by.  What bounds
-// the FP64 kernel now is instruction issue: 54% of the slots, the integer pipe 57% and the FP64 pipe 49%
-// busy.
+// others and works through them, 32 at a time, with the whole scheme in FP64 arithmetic
+// (knp_node): in a node-wide fixed point its weights lose the bits by which one axis lies below the
+// other (rows of unit noise beside rows of 1e-9: increments 2e-10 off, against 1.5e-16).  What is
+// left over, seldom a full warp's worth, goes on the instance's list in global memory when the
+// launch has several waves of blocks (the list lies in the spectrum's buffer, free between the
+// inverse row kernel and the next step's forward one): the warp that completes a chunk of 32 of
+// the list works through it, and the instance's last block takes the rest.  On a launch that the
+// GPU holds at once there are idle lanes to spare, and a tail would cost a scheme's latency: each
+// warp sees to its own.  No barrier follows the tile's loads, so warps at the whole scheme and
+// warps at the short one share the pipes.  A node's result depends on the node alone, not on the
+// lists.  Double words and FP32 take the whole scheme at every node: their long coupled runs
+// amplify any other rounding beyond what two such runs may differ by.
 // body of one block: the tile (tbx, tby) of instance inst, ntiles tiles per instance (the
 // last to start advances the clock); thread (tx_, ty_) of a tx x TY block
 template <typename T, int V, bool GATHER>
@@ -648,7 +647,7 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 node(ln, &x, &y);
                 const size_t o = where(x, y);
                 auto f = [&](int i, int j) -> T { return at(x, y, i, j); };
-                out[o] = fix_node(f, velocity(o, st[y * tpitch + x], f(0, 0)), dt, a.theta_fix, a.time_level);
+                out[o] = knp_node(f, velocity(o, st[y * tpitch + x], f(0, 0)), dt, a.theta, a.theta_code, a.time_level);
             }
             if (c < 0) done += m;
         }

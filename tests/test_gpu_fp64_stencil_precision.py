@@ -51,3 +51,18 @@ def test_limiter_parameter_range(theta, n1, n2):
     smooth = np.sin(2 * np.pi * x + 0.3) * np.cos(2 * np.pi * y + 0.1) + 0.2 * np.sin(4 * np.pi * (x + y) + 1.0)
     for u in (noise, smooth + 1e-3 * noise):
         assert one_step_error(u, theta, 1.0) <= 1e-14
+
+
+@pytest.mark.parametrize("scale", [1e-3, 1e-6, 1e-9, 1e-12])
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("theta,v0", [(1.0, 1.0), (1.7, -1.0), (2.0, 1.0)])
+@pytest.mark.parametrize("n1,n2", [(64, 64), (1024, 256)])
+def test_axes_of_different_size(scale, axis, theta, v0, n1, n2):
+    """Noise of unit size with every fourth line along one axis scaled down: beside such a line the
+    differences along the axis are of unit size, on it they are `scale` times that."""
+    u = np.random.default_rng(12).standard_normal((n2, n1))
+    if axis == 0:
+        u[:, 1::4] *= scale
+    else:
+        u[1::4, :] *= scale
+    assert one_step_error(u, theta, v0) <= 1e-14
