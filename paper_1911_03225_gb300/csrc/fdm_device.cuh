@@ -653,24 +653,6 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
 }
 
 // ---------------------------------------------------------------------------------
-// Nodes of one characteristic direction.  Where both one-sided derivatives along x1 have one
-// sign, and both along x2 have one sign, every pair gives dH/dp of one sign and dH/dq of one
-// sign: one of a+, a- and one of b+, b- is exactly zero, so three of Step 4's four weights are
-// zero, the fourth is one, and that one belongs to the intermediate point whose displacement
-// is zero.  The update is then U - v0 dt |grad| with the gradient (p, q) of that quadrant at
-// the node itself: two reciprocal square roots instead of twelve and a reciprocal, no speeds
-// and no weights, equal to the whole scheme up to the rounding of its weights' ratio.  The limited
-// second differences make both sides' derivatives agree wherever U13 is smooth, its extrema
-// along the axes included: of the coupled random field 99.7% of the nodes qualify at the start
-// and 98% after 150 steps.  An axis along which nothing varies (both derivatives, both limited
-// second differences and the cross differences zero) qualifies as well: its two weights of 1/2
-// belong to equal values.  fix_upwind (fdm_fix.cuh) is this form for FP64 fields.  (FP32: the same
-// skipping took as many instructions as it saved, 69.6 us either way.  Double words: 348 -> 209 us at
-// 2048^2, but a coupled run of 74 steps there amplified the weights' other rounding, 3e-14, to
-// 1e-8, so they keep the whole scheme.)
-// ---------------------------------------------------------------------------------
-
-// ---------------------------------------------------------------------------------
 // Packed FP32 pairs.  Blackwell issues two FP32 additions, multiplications or fused
 // multiply-adds as one instruction (add/sub/mul/fma .rn.f32x2), each lane rounded exactly
 // as the scalar operation.  The FP32 stencil updates two nodes at once in the two lanes:

@@ -5,6 +5,8 @@ Tolerance of one step (relative L2 of the increment): an increment is a sum of a
 products and quotients of the field's differences, on either side; on fields with no exact ties
 each rounds within 2^-53 of the largest, and the fields' differences are of their own size, so 1e-14 (ninety
 times 2^-53) covers both."""
+from math import erf, pi, sqrt
+
 import numpy as np
 import pytest
 
@@ -28,17 +30,21 @@ def _built():
     oracle.set_threads(prev)
 
 
-def one_step_error(u, theta, v0):
+def one_step(u, theta, v0, level=B.T_MIDPOINT):
     n2, n1 = u.shape
-    p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=v0, theta=theta, cfl=0.45, autotune=0)
+    p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=v0, theta=theta, time_level=level, cfl=0.45, autotune=0)
     op = oracle.Params(**{k: getattr(p, k) for k in oracle.Params.__dataclass_fields__})
     ref, rc = oracle.run(op, u, 1, K=np.zeros((n2, n1)))   # the prescribed celerity needs no stress
     assert rc == 0
     with FDM(p) as sim:
         sim.set_plastic_distortion(u)
         sim.step(1)
-        got = sim.read_fields("up13")["up13"]
-    return np.linalg.norm(got - ref.up13) / np.linalg.norm(ref.up13 - u)
+        return sim.read_fields("up13")["up13"], ref.up13
+
+
+def one_step_error(u, theta, v0):
+    got, ref = one_step(u, theta, v0)
+    return np.linalg.norm(got - ref) / np.linalg.norm(ref - u)
 
 
 @pytest.mark.parametrize("theta", [float(np.nextafter(2.0, 0.0)), 2.0 - 1e-10, 2.0 - 1e-9, 1.25,
@@ -66,3 +72,83 @@ def test_axes_of_different_size(scale, axis, theta, v0, n1, n2):
     else:
         u[1::4, :] *= scale
     assert one_step_error(u, theta, v0) <= 1e-14
+
+
+@pytest.mark.parametrize("theta,level,v0", [(1.0, B.T_MIDPOINT, -1.0), (1.7, B.T_MIDPOINT, -1.0),
+                                            (1.0, B.T_LITERAL, 1.0), (1.7, B.T_LITERAL, -1.0)])
+@pytest.mark.parametrize("n1,n2", [(64, 32), (1024, 256)])
+def test_nodes_beside_a_steep_front(theta, level, v0, n1, n2):
+    """Ridges of unit slope over a floor of noise of 1e-9: nodes at their feet have outer neighbours and
+    diagonals 1e9 times their own differences.  On the nodes that move by less than 1e-6 the increments
+    are the floor's own.  Bar 1e-13: with these directions and limiters no term of a foot's increment
+    cancels, and FP64 arithmetic stays within 1.5e-16 of 113 bits."""
+    x, y = np.arange(n1)[None, :], np.arange(n2)[:, None]
+    ridge = np.maximum(0.0, 3.3 - np.abs((x + 0.5 * y) % 16 - 8.2))
+    u = ridge + 1e-9 * np.random.default_rng(13).standard_normal((n2, n1))
+    got, ref = one_step(u, theta, v0, level)
+    floor = np.abs(ref - u) < 1e-6
+    assert floor.mean() > 0.2
+    assert np.linalg.norm((got - ref)[floor]) <= 1e-13 * np.linalg.norm((ref - u)[floor])
+
+
+def annihilation(u, steps, r):
+    """The same scheme on a row that does not vary along x2 (theta = 1, v0 = 1), in the precision of u: the
+    x2 weights are halves of equal values, so each side of the x1 axis has one value."""
+    h = u.dtype.type(0.5)
+    r = u.dtype.type(r)
+
+    def minmod3(a, b, c):
+        lo, hi = np.minimum(np.minimum(a, b), c), np.maximum(np.maximum(a, b), c)
+        return np.where(lo > 0, lo, np.where(hi < 0, hi, 0 * a))
+
+    for _ in range(steps):
+        d = np.roll(u, -1) - u                     # to the next cell
+        m1, m3, p3 = np.roll(d, 1), np.roll(d, 2), np.roll(d, -1)
+        c = d - m1
+        S = (minmod3(p3 - d, h * (p3 - m1), c), minmod3(c, h * (d - m3), m1 - m3))
+        D = (d, m1)
+        P = (D[0] - h * S[0], D[1] + h * S[1])
+        a = np.maximum(0, np.maximum(np.sign(P[0]), np.sign(P[1])))
+        b = np.minimum(0, np.minimum(np.sign(P[0]), np.sign(P[1])))
+        w = np.where(a - b > 0, a - b, 1)
+        weight = (np.where(a - b > 0, -b / w, h), np.where(a - b > 0, a / w, h))
+        inc = 0 * u
+        for s, (e, cx) in enumerate(((a * r, 1), (b * r, -1))):
+            p = D[s] + S[s] * (e - h * cx)
+            p = p - h * r * S[s] * np.sign(p)
+            inc = inc + weight[s] * (e * (D[s] + h * S[s] * (e - cx)) - r * np.abs(p))
+        u = u + inc
+    return u
+
+
+@pytest.mark.skipif(np.finfo(np.longdouble).eps > 2.0 ** -60, reason="needs a wider long double")
+def test_long_run_does_not_drift():
+    """Two walls that annihilate, 200 steps, down to 1e-40 of the start: against the same run in long
+    doubles.  Rounding of the state alone is a random walk of 200 halvings (200^1/2 2^-54 = 8e-16 relative
+    at one node), which the FP64 oracle's distance from that run measures; a bias of 2^-55 in each step
+    would come to 5.6e-15.  Bar: four times the oracle's distance, over four wall pairs together."""
+    n1, n2, steps, cfl = 128, 16, 200, 0.5
+    gpu = cpu = 0.0
+    x = np.arange(n1, dtype=np.float64)
+    for a, b in ((-0.31, 0.12), (0.22, -0.4), (0.47, 0.35), (-0.08, -0.27)):
+        s, sep = 3.0 * (1 + 0.2 * a), n1 / 4.0 * (1 + 0.1 * b)
+        row = np.array([s * sqrt(pi / 2) * (erf((t - n1 / 2 + sep / 2) / (s * sqrt(2)))
+                                            - erf((t - n1 / 2 - sep / 2) / (s * sqrt(2)))) for t in x])
+        u = np.repeat(row[None, :], n2, axis=0)
+        exact = annihilation(row.astype(np.longdouble), steps, cfl)
+        p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=1.0, theta=1.0, cfl=cfl, autotune=0)
+        op = oracle.Params(**{k: getattr(p, k) for k in oracle.Params.__dataclass_fields__})
+        ref, rc = oracle.run(op, u, steps, K=np.zeros((n2, n1)))
+        assert rc == 0
+        with FDM(p) as sim:
+            sim.set_plastic_distortion(u)
+            sim.step(steps)
+            got = sim.read_fields("up13")["up13"]
+        norm = np.linalg.norm(exact.astype(np.float64))
+        assert 0 < norm < 1e-30
+
+        def distance(v):
+            return float(np.sqrt(np.mean([np.sum(((w.astype(np.longdouble) - exact) / norm) ** 2) for w in v])))
+        gpu += distance(got) ** 2
+        cpu += distance(ref.up13) ** 2
+    assert gpu ** 0.5 <= 4 * cpu ** 0.5
