@@ -351,7 +351,10 @@ __global__ void __launch_bounds__(FixBlock<L, false>::most, FixBlock<L, false>::
             to_fixed(x, v, f);
             fix_transform<L, -1>(v, j, c, A + c * ld, B + c * ld, pt2, f.need);
             sc = f.E - 1080 + f.need;
-            if (!symbol || f.nan || f.pre || (packed_block && c == 0)) {
+            // the power stays out of the symbol's products and joins the inverse transform's, where
+            // the two together cannot leave FP64's range (8 FP64 products a thread)
+            const bool apart = a.moderate && sc >= -500 && sc <= 700;
+            if (!symbol || !apart || f.nan || f.pre || (packed_block && c == 0)) {
                 from_fixed<8>(v, x, sc, f);
                 sc = 0;
             } else {

@@ -1128,6 +1128,8 @@ ColArgs<T> col_args(const Dev& d, int mode, bool with_mean, int sym_odd2 = 0, in
     a.frac = (double)d.p.nh / (double)d.p.nz;
     a.xi1_unit = T(6.283185307179586476925286766559 / ((double)d.p.n1 * d.p.dx));
     a.xi2_unit = T(6.283185307179586476925286766559 / ((double)d.p.n2 * d.p.dx));
+    auto mid = [](double v) { return v >= 0x1p-200 && v <= 0x1p200; };
+    a.moderate = mode == COL_K || mode == COL_SYM ? mid(a.mu) : mid((double)a.xi1_unit) && mid((double)a.xi2_unit);
     a.sym_odd2 = sym_odd2;
     a.sym_imag = sym_imag;
     return a;

@@ -108,6 +108,7 @@ struct ColArgs {
     double mu, frac;             // COL_K: shear modulus; the layer's share of the cell
     T xi1_unit, xi2_unit;        // 2 pi / (n dx): xi = k~ * unit
     int sym_odd2, sym_imag;      // COL_SYM: symbol odd in xi2; symbol imaginary
+    int moderate;                // the symbol's unit (mu, xi) lies in [2^-200, 2^200]
 };
 
 template <typename T>
