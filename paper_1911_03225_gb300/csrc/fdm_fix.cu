@@ -89,16 +89,20 @@ __device__ __forceinline__ unsigned mag_of(const cpx<double>* x) {
     for (int u = 0; u < 8; ++u) m = max(m, max(fix_mag(x[u].x), fix_mag(x[u].y)));
     return m;
 }
-// eight values in the sequence's units; the branches for its rare scales keep their products
-// off the common path
-__device__ __forceinline__ void to_fixed(cpx<double>* x, cfx* v, const FixScale& f) {
+// eight values in the sequence's units, and, if asked for, what their rounding left (fix_from_lost);
+// the branch for its rare scales keeps their products off the common path
+template <bool LOST = false>
+__device__ __forceinline__ void to_fixed(cpx<double>* x, cfx* v, const FixScale& f, int* lost = nullptr) {
     if (f.pre) {
         const double p = f.pre > 0 ? kUp : kDown;
 #pragma unroll
         for (int u = 0; u < 8; ++u) x[u] = mk(x[u].x * p, x[u].y * p);
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = mkx(fix_from(x[u].x, f.E), fix_from(x[u].y, f.E));
+    for (int u = 0; u < 8; ++u) {
+        if constexpr (LOST) v[u] = mkx(fix_from_lost(x[u].x, f.E, *lost), fix_from_lost(x[u].y, f.E, *lost));
+        else v[u] = mkx(fix_from<kFixBits, true>(x[u].x, f.E), fix_from<kFixBits, true>(x[u].y, f.E));
+    }
 }
 // N results as doubles: integers that carry the scale sc (the sequence's units included)
 template <int N> __device__ __forceinline__ void from_fixed(const cfx* v, cpx<double>* x, int sc, const FixScale& f) {
@@ -172,7 +176,8 @@ constexpr size_t fix_max_smem(int L, bool rows) {   // of any R
 
 // ------------------------------------------------------------------ row forward (R2C)
 // grid (n2 / R, instances); see row_forward_kernel.  The row's sum (for <U13>) is taken from
-// the integers, exactly, and rounded once per thread.
+// the integers and what their rounding left, to 2^-64 of the row's largest value each, and rounded
+// once per thread.
 template <int L>
 __global__ void __launch_bounds__(FixBlock<L, true>::most, FixBlock<L, true>::minb)
     fix_row_forward_kernel(const double* src0, const double* src1, cpx<double>* spec, int n2, int R,
@@ -203,12 +208,13 @@ __global__ void __launch_bounds__(FixBlock<L, true>::most, FixBlock<L, true>::mi
             x[u] = on ? src[(size_t)(y0 + row) * L + j + u * T] : mk(0.0, 0.0);
         const FixScale f = seq_scale<T>(mag_of(x), row, tid, s_stat, log2i(T));
         cfx v[8];
-        to_fixed(x, v, f);
+        int lost = 0;
+        to_fixed<true>(x, v, f, &lost);
         if (row_partials) {
             long long s = 0;   // |components| <= 2^58: 16 of them fit
 #pragma unroll
             for (int u = 0; u < 8; ++u) s += v[u].x + v[u].y;
-            double d = (double)s;
+            double d = (double)s + (double)lost * 0x1p-6;
 #pragma unroll
             for (int o = (T < 32 ? T : 32) / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
             if ((tid & 31) == 0) s_sum[tid >> 5] = d;

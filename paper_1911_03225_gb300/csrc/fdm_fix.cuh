@@ -5,7 +5,7 @@
 // of FP64 data needs no floating point: its error is a fraction of the sequence's largest
 // value whatever the format, so a sequence whose largest magnitude is 2^(e+1) is held as
 // integers in units of 2^(e+1-58) (an exact shift of every mantissa for values within 2^-5 of
-// the largest, and a truncation five bits below FP64's own rounding of the largest for the
+// the largest, and rounded to nearest five bits below FP64's own rounding of the largest for the
 // others), transformed with integer additions and 62-bit twiddles, and converted back with one
 // rounding.  Every pass shifts right by the bits it may grow, inside the twiddle product, so
 // nothing overflows.  Measured against long-double transforms the result is closer than an
@@ -203,6 +203,23 @@ template <int B = kFixBits, bool NEAR = false> FIX_HD long long fix_from(double 
 #endif
     if (NEAR) m = (m + 1) >> 1;
     const long long s = (long long)u >> 63;
+    return ((long long)m ^ s) - s;
+}
+// fix_from<kFixBits, true>(x, E); adds what its rounding left of x, in units of 2^-6 of its units, to
+// lost (six bits of it: to 2^-64 of 2^E)
+FIX_HD long long fix_from_lost(double x, int E, int& lost) {
+    const unsigned long long u = fix_bits(x);
+    const int d = E - ((int)(u >> 52) & 0x7ff);
+    unsigned long long m = ((u & 0xfffffffffffffull) | 0x10000000000000ull) << (kFixBits - 53 + 6);
+#if defined(__CUDA_ARCH__)
+    asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(d));   // 0 beyond 63
+#else
+    m = d > 63 ? 0 : m >> d;
+#endif
+    const int s = (int)(u >> 32) >> 31;
+    const int l = (int)((unsigned)m << 26) >> 26;
+    lost += (l ^ s) - s;
+    m = (m + 32) >> 6;
     return ((long long)m ^ s) - s;
 }
 // a 2^sc as a double, one rounding (sc keeps every a != 0 in the normal range)

@@ -3,6 +3,8 @@ range, where the field and the elastic modulus are both small or both large.
 
 Tolerance (relative L2): every scale is a power of two, so the solve is the one at unit scale but
 for results below the normal range, a 2^-60 part here; 1e-14 as for the transforms at unit scale."""
+import math
+
 import numpy as np
 import pytest
 
@@ -42,3 +44,22 @@ def test_static_solve_small_and_large_modulus(kind, n1, n2, field_exp, modulus_e
         got = sim.read_fields("tau13")["tau13"]
     got = np.ldexp(got, -(field_exp + modulus_exp))
     assert np.linalg.norm(got - ref) <= 1e-14 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n1", [64, 512, 2048, 4096])
+@pytest.mark.parametrize("background", ["random", "constant"])
+def test_mean_of_rows_of_unequal_size(n1, background):
+    """The mean of U13 sets the stress under a strain: a field of equal rows, one value of 1 and positive
+    ones of 2^-20 and less, in a full-depth layer (no other stress).  Bar: eight roundings of 2^-53 (a thread's
+    and the row's sum, the mean, the loading law's products and difference, the way back to doubles)."""
+    r = np.random.default_rng(n1).uniform(0.0, 2.0 ** -20, n1)
+    if background == "constant":
+        r[:] = r[0]
+    r[n1 // 3] = 1.0
+    p = Params(n1=n1, n2=16, nz=16, nh=16, velocity_mode=B.V_STRESS, loading_mode=B.LOAD_STRAIN_RAMP, autotune=0)
+    with FDM(p) as sim:
+        sim.set_plastic_distortion(np.repeat(r[None, :], 16, axis=0))
+        sim.static_solve()
+        tau = sim.read_fields("tau13")["tau13"]
+    want = -p.E / (2 * (1 + p.nu)) * (math.fsum(r) / n1)
+    assert np.abs(tau / want - 1.0).max() <= 8 * 2.0 ** -53
