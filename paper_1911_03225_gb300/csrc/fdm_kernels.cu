@@ -637,7 +637,7 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
                 } else {
                     const unsigned k = __ldcg(glist + (size_t)c * kRound + i);
                     *x = (int)(k & (unsigned)(n1 - 1));
-                    *y = (int)(k / (unsigned)n1);
+                    *y = (int)(k / (unsigned)n1) & (n2 - 1);   // in the field whatever the entry
                 }
             };
             auto at = [&](int x, int y, int i, int j) -> T { return u[((y + j) & my) * pitch + ((x + i) & mx)]; };
@@ -1216,6 +1216,8 @@ KnpArgs<T> knp_args(const Dev& d) {
     a.sc = d.sc;
     a.gated = d.gated;
     const size_t n = (size_t)d.p.n1 * d.p.n2;
+    // the lists lie in the spectra, which the next step's forward rows overwrite: those may not start
+    // before every warp of the stencil is done with its entries (launch_phase)
     a.list = static_cast<unsigned*>(d.spec);
     a.list_stride = n * sizeof(T) / sizeof(unsigned);
     a.chunks = d.chunks;
@@ -1234,7 +1236,10 @@ void launch_knp(const Dev& d, cudaStream_t s) {
 }
 
 // one kernel of a step for every instance of the group (Sec. 3.1.1: static solve with U^n,
-// then transport); U^n is buffer sc[i].cur of instance i
+// then transport); U^n is buffer sc[i].cur of instance i.  Each kernel waits for the whole of the one
+// before it: plain launches on one stream.  The FP64 stencil's lists count on it (they lie in the
+// spectra, and a warp reads its entries up to the kernel's end), so a launch that lets the next
+// step's forward rows start early needs the lists in a place of their own.
 template <typename T>
 void launch_phase(const Dev& d, int phase, cudaStream_t s) {
     cpx<T>* spec = (cpx<T>*)d.spec;
