@@ -66,14 +66,16 @@ def bytes_per_cell(elt, pair=False):
 #   v0 dt and v0 dt / 2 2; the row and column quadratics of the two sides 20 + 20;
 #   four corners of 36 (mixed difference 3, value 5, gradient 4, midpoint predictor 15,
 #   |grad| 5, Psi and its weight 4) 144; projection 5.  Total 250, of which 11 reciprocal
-#   square roots and one reciprocal.  The mixed path does all of them at every node; the FP64 and
-#   double-word paths take a shorter form where one characteristic direction leaves three quadrants
-#   without weight, FP64 in integers, so no flop count of theirs compares with a flop rate.
+#   square roots and one reciprocal.  The mixed and the double-word path do all of them at every
+#   node.  FP64 takes a shorter form, in integers, where one characteristic direction leaves three
+#   quadrants without weight, so no flop count of its own compares with a flop rate.
 KNP_FLOPS_PER_CELL = 250
+# the measured arithmetic rate that bounds a precision's stencil (measured_arith_peaks)
+STENCIL_PEAK = {"mixed": ("fp32", "FP32"), "df64": ("df64", "double-word")}
 
 
-KERNEL_SOURCES = ["fdm_kernels.cu", "fdm_fix.cu", "fdm_f32.cu", "fdm_step.cuh", "fdm_fix.cuh", "fdm_device.cuh", "fdm_df.cuh",
-                  "fdm_internal.h"]
+KERNEL_SOURCES = ["fdm_kernels.cu", "fdm_fix.cu", "fdm_f32.cu", "fdm_step.cuh", "fdm_fix.cuh", "fdm_device.cuh",
+                  "fdm_df.cuh", "fdm_internal.h"]
 
 
 def kernel_source_hash():
@@ -302,17 +304,18 @@ def run_ours(args, world, rank, local):
     value = cells * K * world / (r["total_ms"] / 1e3)
 
     def roofline(prec, rr):
-        """Roofline of the step's dominant kernel: the mixed path's stencil against the measured
-        multiply-add rate of its arithmetic (it is bound by arithmetic, not by HBM), everything
-        else against the HBM peak."""
+        """Roofline of the step's dominant kernel: the mixed and double-word paths' stencils against
+        the measured multiply-add rate of their arithmetic (they are bound by it, not by HBM),
+        everything else against the HBM peak."""
         d = rr["dominant"]
         d_ms = rr["phase_ms"][d]
         hbm_gbs = rr["bpc"][d] * cells / (d_ms / 1e3) / 1e9
-        if d == "knp_step" and prec == "mixed":
-            rl = {"bound": "alu", "achieved": KNP_FLOPS_PER_CELL * cells / (d_ms / 1e3) / 1e9, "peak": peaks["fp32"],
+        if d == "knp_step" and prec in STENCIL_PEAK:
+            key, name = STENCIL_PEAK[prec]
+            rl = {"bound": "alu", "achieved": KNP_FLOPS_PER_CELL * cells / (d_ms / 1e3) / 1e9, "peak": peaks[key],
                   "unit": "GFLOP/s", "flops_per_cell": KNP_FLOPS_PER_CELL,
-                  "peak_source": "measured in this run (of measured): FP32 multiply-add chains on every SM, "
-                                 "fdm_measure_arith_rate, SM clock %s MHz" % peaks["clocks"].get("sm_mhz")}
+                  "peak_source": "measured in this run (of measured): %s multiply-add chains on every SM, "
+                                 "fdm_measure_arith_rate, SM clock %s MHz" % (name, peaks["clocks"].get("sm_mhz"))}
         else:
             rl = {"bound": "hbm", "achieved": hbm_gbs, "peak": hbm_peak, "unit": "GB/s", "peak_source": peak_src}
         rl["frac"] = rl["achieved"] / rl["peak"]
