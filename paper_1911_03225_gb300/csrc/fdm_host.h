@@ -4,6 +4,7 @@
 #pragma once
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "fdm_internal.h"
@@ -79,7 +80,9 @@ inline bool geometry_from_config(const fdm_params& p, const fdm_launch_config& c
     for (int k = 0; k < kKnpShapes && shape < 0; ++k) {
         int ty, npt, minb;
         knp_shape_info<T>(k, &ty, &npt, &minb);
-        if (ty == c.stencil_block_rows && npt == c.stencil_nodes && minb == c.stencil_min_blocks) shape = k;
+        // FP64's shapes of 256 threads were named by 2 while they were compiled for two blocks per SM
+        const bool former = std::is_same<T, double>::value && minb == 4 && c.stencil_min_blocks == 2;
+        if (ty == c.stencil_block_rows && npt == c.stencil_nodes && (minb == c.stencil_min_blocks || former)) shape = k;
     }
     if (!r_ok || !c_ok || shape < 0) return false;
     *g = geometry<T>(p.n1, p.n2, c.rows_per_block, c.cols_per_block, shape);

@@ -370,9 +370,12 @@ template <> struct KnpShapes<float> {   // nodes are updated two at a time (pack
     static constexpr int ty[kKnpShapes] = {8, 8, 16, 8}, npt[kKnpShapes] = {4, 2, 2, 4},
                          minb[kKnpShapes] = {4, 4, 1, 3};
 };
+// FP64: four blocks of 256 threads (64 registers, some spilled), since the short form waits on long
+// integer chains (2048^2, random field after 30 steps: 343 us with two, 286 with three, 265 with
+// four, 262 with five)
 template <> struct KnpShapes<double> {
     static constexpr int ty[kKnpShapes] = {8, 8, 16, 8}, npt[kKnpShapes] = {2, 1, 1, 4},
-                         minb[kKnpShapes] = {2, 2, 1, 2};
+                         minb[kKnpShapes] = {4, 4, 1, 4};
 };
 template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed FP32 pairs)
     static constexpr int ty[kKnpShapes] = {8, 8, 16, 8}, npt[kKnpShapes] = {2, 4, 2, 2},
@@ -392,8 +395,9 @@ template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed 
 // GPU holds at once there are idle lanes to spare, and a tail would cost a scheme's latency: each
 // warp sees to its own.  No barrier follows the tile's loads, so warps at the whole scheme and
 // warps at the short one share the pipes.  A node's result depends on the node alone, not on the
-// lists.  Double words and FP32 take the whole scheme at every node: their long coupled runs
-// amplify any other rounding beyond what two such runs may differ by.
+// lists.  2048^2, random field after 30 steps: 1388 us with the whole scheme at every node, 265 with
+// the lists; bound by instruction issue.  Double words and FP32 take the whole scheme at every node:
+// their long coupled runs amplify any other rounding beyond what two such runs may differ by.
 // body of one block: the tile (tbx, tby) of instance inst, ntiles tiles per instance (the
 // last to start advances the clock); thread (tx_, ty_) of a tx x TY block
 template <typename T, int V, bool GATHER>
@@ -654,19 +658,12 @@ __device__ __forceinline__ void knp_step_body(const T* phi0, const T* phi1, cons
     }
 }
 
-// Blocks per SM the kernel is compiled for: the shape's own figure; in FP64 four of 256 threads (64
-// registers, some spilled), whose forms wait on long integer chains (2048^2 random field: 327 us
-// with two, 272 with three, 241 with four, 238 with five)
-template <typename T, int V> constexpr int knp_blocks() {
-    return std::is_same<T, double>::value && KnpShapes<T>::ty[V] == 8 ? 4 : KnpShapes<T>::minb[V];
-}
-
 template <typename T, int V, bool GATHER>
-__global__ void __launch_bounds__(TX * KnpShapes<T>::ty[V], knp_blocks<T, V>())
+__global__ void __launch_bounds__(TX * KnpShapes<T>::ty[V], KnpShapes<T>::minb[V])
     knp_step_kernel(const T* phi0, const T* phi1, const T* __restrict__ tau0, int n1, int n2, int npt,
                     KnpArgs<T> a) {
-    knp_step_body<T, V, GATHER>(phi0, phi1, tau0, n1, n2, npt, a, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x * gridDim.y,
-                        threadIdx.x, threadIdx.y, blockDim.x);
+    knp_step_body<T, V, GATHER>(phi0, phi1, tau0, n1, n2, npt, a, blockIdx.x, blockIdx.y, blockIdx.z,
+                                gridDim.x * gridDim.y, threadIdx.x, threadIdx.y, blockDim.x);
 }
 
 // ------------------------------------------------------------------ set-up / readout helpers
@@ -996,7 +993,9 @@ template <typename T> static size_t fft_block_smem(int nseq, int L) {
 }
 
 // R rows per row-kernel block is valid when R <= n2, R <= 16, R n1/2 <= 8 x the thread
-// bound (one radix-8 butterfly per thread) and the rows fit the shared-memory limit
+// bound (one radix-8 butterfly per thread) and the rows fit the shared-memory limit: the generic
+// kernels' conditions, and the shapes offered for every type.  The FP64 and mixed kernels work
+// through a block's R rows (C columns) a few at a time and fit any of them.
 template <typename T> static bool row_ok(int n1, int n2, int R) {
     return R <= n2 && R <= 16 && R * (n1 / 2) <= 8 * FftBounds<T>::threads &&
            fft_block_smem<T>(R, n1 / 2) <= kMaxDynSmem;
@@ -1526,9 +1525,9 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
                     } else if (phase == 2) {
                         row_inverse_body<float>(G.spec, G.tau, G.n1, G.n2, G.R, G.tw1, G.pt1, G.row, tile, inst, per);
                     } else {
-                        knp_step_body<float, kPersistShape, false>(G.phi0, G.phi1, G.tau, G.n1, G.n2, G.knp_npt, G.knp,
-                                                            tile % G.knp_gx, tile / G.knp_gx, inst, per,
-                                                            threadIdx.x & (TX - 1), threadIdx.x / TX, TX);
+                        knp_step_body<float, kPersistShape, false>(G.phi0, G.phi1, G.tau, G.n1, G.n2, G.knp_npt,
+                                                                   G.knp, tile % G.knp_gx, tile / G.knp_gx, inst, per,
+                                                                   threadIdx.x & (TX - 1), threadIdx.x / TX, TX);
                     }
                     __syncthreads();   // the next task reuses the block's shared memory
                 }
