@@ -9,8 +9,8 @@
 //
 // What bounds them: instruction issue (about 250 instructions per complex point and transform,
 // half of them 64-bit additions), no longer the FP64 pipe, which keeps the conversions to
-// double.  2048^2, one launch, FP64 -> fixed point: rows 190 -> 44 us, column pass 303 -> 88
-// us, inverse rows 190 -> 59 us; 1024^2: 52 -> 17, 94 -> 32, 55 -> 25 us.
+// double.  2048^2, one launch (events between the kernels), FP64 -> fixed point: rows 190 -> 50 us,
+// column pass 303 -> 88, inverse rows 190 -> 64; 1024^2: 52 -> 21, 94 -> 39, 55 -> 27.
 #include <type_traits>
 
 #include "fdm_fix.cuh"
@@ -142,7 +142,7 @@ __device__ __forceinline__ void fix_transform(cfx* v, int j, int seq, cfx* A, cf
 
 __host__ __device__ constexpr int log2i(int v) { return v <= 1 ? 0 : 1 + log2i(v / 2); }
 // threads of a block: enough sequences for a full warp and up to 256 threads, three blocks per
-// SM (80 registers, a few spilled: 44 us for the rows of 2048^2 against 51 with two blocks of
+// SM (80 registers, a few spilled: the rows of 2048^2 took 44 us so and 51 with two blocks of
 // 128); 512 where one row takes 256, because the transposed accesses need two rows for 32-byte
 // segments, and where one column takes 512
 template <int L, bool ROWS> struct FixBlock {
@@ -181,7 +181,8 @@ constexpr size_t fix_max_smem(int L, bool rows) {   // of any R
 template <int L>
 __global__ void __launch_bounds__(FixBlock<L, true>::most, FixBlock<L, true>::minb)
     fix_row_forward_kernel(const double* src0, const double* src1, cpx<double>* spec, int n2, int R,
-                           const twx* __restrict__ tw1, const twx* __restrict__ pt1, double* row_partials, InstCtl ctl) {
+                           const twx* __restrict__ tw1, const twx* __restrict__ pt1, double* row_partials,
+                           InstCtl ctl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_run, s_cur;
     __shared__ WarpStat s_stat[16];
@@ -392,7 +393,8 @@ __global__ void __launch_bounds__(FixBlock<L, false>::most, FixBlock<L, false>::
                             const double p = 0.5 * (m0.y + mN.y), d = 0.5 * (m0.y - mN.y);
                             x[u] = mk(d * zr.y - p * z.y, p * z.x + d * zr.x);
                         }
-                        if (ky == 0 && a.mode == COL_K) x[u].x = 0.0;   // the macroscopic stress: see fix_row_inverse_kernel
+                        // the macroscopic stress: see fix_row_inverse_kernel
+                        if (ky == 0 && a.mode == COL_K) x[u].x = 0.0;
                     }
                 }
                 __syncthreads();

@@ -249,7 +249,9 @@ template <int L> struct FixPlan {
     static __host__ __device__ constexpr int off(int p) { return p == 0 ? 0 : off(p - 1) + 7 * ns(p - 1); }
     // bits that pass p shifts right before its butterflies when `used` of the sequence's
     // `need` bits have been shifted before it
-    static __host__ __device__ constexpr int most(int p) { return p == 0 ? 0 : (radix(p) == 8 ? 3 : (radix(p) == 4 ? 2 : 1)); }
+    static __host__ __device__ constexpr int most(int p) {
+        return p == 0 ? 0 : (radix(p) == 8 ? 3 : (radix(p) == 4 ? 2 : 1));
+    }
     static __host__ __device__ constexpr int before(int p) { return p == 0 ? 0 : 3 * (p - 1); }
     static FIX_HD int shift(int p, int need) {
         const int left = need - before(p);
@@ -359,7 +361,8 @@ FIX_HD long long fix_mulhi2(long long a, long long b, long long c, long long d, 
     fix_halves(c, ch, cl);
     fix_halves(d, dh, dl);
     const long long t = fix_mad(ch, dh, fix_wide(ah, bh));
-    const long long q = fix_mad(cl, dh, fix_mad(ch, dl, fix_mad(al, bh, fix_mad(ah, bl, (long long)(0x80000000u >> s)))));
+    const long long half = (long long)(0x80000000u >> s);
+    const long long q = fix_mad(cl, dh, fix_mad(ch, dl, fix_mad(al, bh, fix_mad(ah, bl, half))));
     return fix_combine(t, q, s);
 }
 // ---- cos(x / beta) for the lattice friction.  x becomes a fraction of a turn first: x / (2 pi beta)
@@ -385,7 +388,7 @@ inline FixTurns fix_turns(double beta) {
     t.e = k - 1022;
     return t;
 }
-// cos(x / beta) in units of 2^-62, within 2^-59; false beyond 2^10 turns (there cos() of the
+// cos(x / beta) in units of 2^-62, within 2^-58; false beyond 2^10 turns (there cos() of the
 // rounded x / beta is further than 1e-12 off, and its own bits are kept), infinities and NaN
 FIX_HD bool fix_cos(double x, const FixTurns& t, long long* c) {
     const unsigned long long u = fix_bits(x);

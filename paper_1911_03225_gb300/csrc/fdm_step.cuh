@@ -217,9 +217,9 @@ template <typename T> VelLaw<T> make_vel(const fdm_params& p, const void* mfac =
 }
 
 // cos(x / beta).  FP64 instructions are what a friction node costs (two lanes per SM): cos() and
-// the division are about 45 of them, fix_cos two and 170 integer ones.  512 x 256 in FP64: rows
-// inverse 34.9 us and stencil 42.2 with cos(), 27.8 and 28.1 with fix_cos (18 and 25 without
-// friction).  The other paths keep cos(), whose roundings their long runs amplify.
+// the division are about 45 of them, fix_cos two and 170 integer ones.  512 x 256 in FP64 with
+// mobility factors: rows inverse 41.0 us and stencil 47.2 with cos(), 32.8 and 43.0 with fix_cos (22.5
+// and 38.9 without friction).  The other paths keep cos(), whose roundings their long runs amplify.
 template <typename T> __device__ __forceinline__ double friction_cos(const VelLaw<T>& v, double x) {
     if constexpr (std::is_same<T, double>::value) {
         long long c;
