@@ -322,19 +322,20 @@ FIX_HD void fix_c2r(cfx xk, cfx xc, twx w, cfx* zk, cfx* zc) {
 // as it saved, 69.6 us either way.  Double words: 348 -> 209 us at 2048^2, but a coupled run of 74
 // steps there amplified the weights' other rounding, 3e-14, to 1e-8, so they keep the whole scheme.)
 //
-// The first differences are FP64 subtractions; from there the node works in units of 2^-57 of 2^E
+// The first differences are FP64 subtractions; from there the node works in units of 2^-59 of 2^E
 // (half units from the derivatives on), rounded to nearest, with 2^E the bound of the four
 // differences to its neighbours.  The differences beyond those enter through the limiter alone,
 // which caps what they contribute: where they are larger they are set to 8 times the bound, so the
 // tail of a front keeps its own scale.  (One scale over all of them, and shifts that round down,
 // left each step of such a tail 2^-55 off: 5.6e-15 after 200 steps of two walls that annihilate down
-// to 1e-42, against 2.4e-16 to 7.3e-16 for FP64 arithmetic; 2.1e-16 to 7.1e-16 now.)  A node whose
-// side's differences lie below 2^-4 of the bound would keep fewer bits than FP64's, one whose
-// derivatives lie within the rounding may have the wrong sign: both are left to the whole scheme.
-// Against 113-bit arithmetic, error of the increment in units of 2^-53, 99.9% of the nodes below:
-// noise 2.6 (FP64 arithmetic: 16), smooth with noise 1.9 (3.6), tails 1.3 (4.2), kinks 2.1 (3.6),
-// axes of different size 1.8 (3.2), exponents spread over 60 bits, where either cancels, 3e6 (7e6).
-// Integer instructions and 13 FP64 ones per node replace 39 FP64 ones.
+// to 1e-42, against 2.4e-16 to 7.3e-16 for FP64 arithmetic; 2.7e-17 to 4.2e-16 now; with two bits
+// fewer 2.1e-16 to 7.1e-16.)  A node whose side's differences lie below 2^-6 of the bound would keep
+// fewer bits than FP64's, one whose derivatives lie within the rounding may have the wrong sign:
+// both are left to the whole scheme. Against 113-bit arithmetic, error of the increment in units of
+// 2^-53, 99.9% of the nodes below: noise 2.6 (FP64 arithmetic: 16), smooth with noise 1.9 (3.6),
+// tails 1.3 (4.2), kinks 2.1 (3.6), axes of different size 1.8 (3.2), exponents spread over 60 bits,
+// where either cancels, 7e5 (5e6). Integer instructions and 13 FP64 ones per node replace 39 FP64
+// ones.
 // ---------------------------------------------------------------------------------
 // (a b) / 2^64 rounded (the product of the low halves left out), |a|, |b| <= 2^62 (fix_halves
 // rounds up: it needs 2^31 of room below 2^63)
@@ -431,12 +432,11 @@ FIX_HD bool fix_cos(double x, const FixTurns& t, long long* c) {
     return true;
 }
 // of one sign and none zero: the one of least magnitude, else 0
-FIX_HD long long fix_minmod3(long long a, long long b, long long c) {
+FIX_HD long long fix_minmod(long long a, long long b) {
     const long long s = a >> 63;
     long long m = a ^ s;
-    const long long mb = b ^ s, mc = c ^ s;   // negative where the signs differ (or zero meets a negative)
+    const long long mb = b ^ s;   // negative where the signs differ (or zero meets a negative)
     m = mb < m ? mb : m;
-    m = mc < m ? mc : m;
     return (m ^ s) & ~(m >> 63);
 }
 // the limiter parameter theta in [1, 2]: code 1 or 2 when it is exactly that, else 2^-3 theta as
@@ -491,15 +491,15 @@ FIX_HD long long fix_rsqrt(long long x) {
     const int c = fix_round(s * (0.375f * ef) * ef * 0x1p61f);
     return fix_mad(c, 1, ((long long)y << 32) + d);
 }
-// (p, q) shifted left by *L so that the larger has 61 bits, and |(p, q)|^2 of those / 2^64, in
-// [2^56, 2^59); false for (0, 0)
+// (p, q) shifted left by *L (right where it is negative: 62 bits and more) so that the larger has 61
+// bits, and |(p, q)|^2 of those / 2^64, in [2^56, 2^59); false for (0, 0)
 FIX_HD bool fix_norm2(long long p, long long q, long long* ps, long long* qs, int* L, long long* r2) {
     const long long sp = p >> 63, sq = q >> 63;
     const long long m = ((p ^ sp) - sp) | ((q ^ sq) - sq);
     if (m == 0) return false;
     *L = fix_clz(m) - 3;
-    *ps = (long long)((unsigned long long)p << *L);
-    *qs = (long long)((unsigned long long)q << *L);
+    *ps = *L < 0 ? p >> -*L : (long long)((unsigned long long)p << *L);
+    *qs = *L < 0 ? q >> -*L : (long long)((unsigned long long)q << *L);
     int ph, pl, qh, ql;
     fix_halves(*ps, ph, pl);
     fix_halves(*qs, qh, ql);
@@ -509,8 +509,8 @@ FIX_HD bool fix_norm2(long long p, long long q, long long* ps, long long* qs, in
     return true;
 }
 
-// four more than FP64's: first differences down to 2^-4 of the bound stay exact
-constexpr int kNodeBits = 57;
+// six more than FP64's: differences down to 2^-6 of the bound stay exact
+constexpr int kNodeBits = 59;
 // a difference beyond the first ones, in their units: |result| <= 8 times their bound, which it is
 // set to if it lies above
 FIX_HD long long fix_outer(double x, int E) {
@@ -550,13 +550,15 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
     if ((turn_x && (int)(mx >> 20) > E + 3) || (turn_y && (int)(my >> 20) > E + 3)) return false;
     const long long dxm3 = fix_outer(axm3, E), dxp3 = fix_outer(axp3, E);
     const long long dym3 = fix_outer(aym3, E), dyp3 = fix_outer(ayp3, E);
-    // the limited second differences: the minima of doubles, halved to nearest
-    auto half = [](long long a) { return (a + 1) >> 1; };
-    const long long cx2 = fix_theta(dxp1 - dxm1, th) << 1, cy2 = fix_theta(dyp1 - dym1, th) << 1;
-    const long long Sx0 = half(fix_minmod3(fix_theta(dxp3 - dxp1, th) << 1, dxp3 - dxm1, cx2));
-    const long long Sx1 = half(fix_minmod3(cx2, dxp1 - dxm3, fix_theta(dxm1 - dxm3, th) << 1));
-    const long long Sy0 = half(fix_minmod3(fix_theta(dyp3 - dyp1, th) << 1, dyp3 - dym1, cy2));
-    const long long Sy1 = half(fix_minmod3(cy2, dyp1 - dym3, fix_theta(dym1 - dym3, th) << 1));
+    // the limited second differences of theta a, (a + b) / 2 and theta b: the minima of doubles, halved
+    // to nearest
+    auto limited = [&](long long a, long long b) {
+        const long long m = fix_minmod(fix_theta(fix_minmod(a, b), th) << 1, a + b);
+        return (m + 1) >> 1;
+    };
+    const long long cx = dxp1 - dxm1, cy = dyp1 - dym1;
+    const long long Sx0 = limited(dxp3 - dxp1, cx), Sx1 = limited(cx, dxm1 - dxm3);
+    const long long Sy0 = limited(dyp3 - dyp1, cy), Sy1 = limited(cy, dym1 - dym3);
     // twice the one-sided derivatives, in half units from here on
     const long long px0 = (dxp1 << 1) - Sx0, px1 = (dxm1 << 1) + Sx1;
     const long long qy0 = (dyp1 << 1) - Sy0, qy1 = (dym1 << 1) + Sy1;
@@ -572,11 +574,11 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
     long long p = s0 ? px0 : px1, q = t0 ? qy0 : qy1, ps, qs, r2;
     const long long Dx = s0 ? dxp1 : dxm1, Dy = t0 ? dyp1 : dym1;
     long long Sx = s0 ? Sx0 : Sx1, Sy = t0 ? Sy0 : Sy1;
-    // half units, 2^-58 of the bound, are to stay below 2^-54 of what the gradient is formed from
-    if ((mag(Dx << 1) | mag(Sx) | mag(Dy << 1) | mag(Sy)) < (1ll << (kNodeBits - 3))) return false;
-    const int cx = s0 ? 1 : -1, cy = t0 ? 1 : -1;
+    // half units, 2^-60 of the bound, are to stay below 2^-54 of what the gradient is formed from
+    if ((mag(Dx << 1) | mag(Sx) | mag(Dy << 1) | mag(Sy)) < (1ll << (kNodeBits - 5))) return false;
+    const int ix = s0 ? 1 : -1, iy = t0 ? 1 : -1;
     const double fy = t0 ? yp : ym;
-    const double ac = f(cx, cy) - fy;
+    const double ac = f(ix, iy) - fy;
     const int ea = (int)(fix_mag(ac) >> 20);
     long long fx = s0 ? dxp1 : -dxm1;
     int Ec = E;
@@ -594,7 +596,7 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
     }
     const long long mixed = fix_from<kNodeBits + 2, true>(ac, Ec + 2) - fx;
     if (flat_x || flat_y) {
-        const double oc = flat_y ? f(cx, -cy) - (t0 ? ym : yp) : f(-cx, cy) - fy;   // the other quadrant's
+        const double oc = flat_y ? f(ix, -iy) - (t0 ? ym : yp) : f(-ix, iy) - fy;   // the other quadrant's
         if ((int)(fix_mag(oc) >> 20) > E + 2) return false;
         if (mixed != 0 || fix_from<kNodeBits + 2, true>(oc, E + 2) != (flat_y ? fx : -fx)) return false;
     }
@@ -608,8 +610,8 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
         p -= fix_mulhi(fix_mulhi2(Sx, c, cross, s, 4), h, 2);
         q -= fix_mulhi(fix_mulhi2(cross, c, Sy, s, 4), h, 2);
     }
-    // (|p|, |q| < 2^60.7 for any first differences, diagonal and |v0 dt / h| <= 1)
-    if (wide && (mag(p) | mag(q)) < (1ll << (kNodeBits - 3))) return false;
+    // (|p|, |q| < 2^62.6 for any first differences, diagonal and |v0 dt / h| <= 1)
+    if (wide && (mag(p) | mag(q)) < (1ll << (kNodeBits - 5))) return false;
     double g = 0.0;   // h |grad|
     if (fix_norm2(p, q, &ps, &qs, &L, &r2)) {
         // |(p 2^L, q 2^L)| = 2^61 sqrt(xi), xi = r2 2^-58, sqrt(xi) = xi / sqrt(xi)

@@ -395,7 +395,7 @@ template <> struct KnpShapes<df> {   // nodes are updated two at a time (packed 
 // GPU holds at once there are idle lanes to spare, and a tail would cost a scheme's latency: each
 // warp sees to its own.  No barrier follows the tile's loads, so warps at the whole scheme and
 // warps at the short one share the pipes.  A node's result depends on the node alone, not on the
-// lists.  2048^2, random field after 30 steps: 1388 us with the whole scheme at every node, 265 with
+// lists.  2048^2, random field after 30 steps: 1388 us with the whole scheme at every node, 269 with
 // the lists; bound by instruction issue.  Double words and FP32 take the whole scheme at every node:
 // their long coupled runs amplify any other rounding beyond what two such runs may differ by.
 // body of one block: the tile (tbx, tby) of instance inst, ntiles tiles per instance (the
