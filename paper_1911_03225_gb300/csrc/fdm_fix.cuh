@@ -580,38 +580,38 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
     const double fy = t0 ? yp : ym;
     const double ac = f(ix, iy) - fy;
     const int ea = (int)(fix_mag(ac) >> 20);
-    long long fx = s0 ? dxp1 : -dxm1;
-    int Ec = E;
-    const bool wide = ea > E + 2;   // the tail of a front: the diagonal dwarfs the axes and sets the units
-    if (wide) {
-        const int k = ea - E - 2;
-        if (k > 30 || flat_x || flat_y) return false;
-        auto down = [&](long long v) { return (v + ((1ll << k) >> 1)) >> k; };
-        Ec = E + k;
-        p = down(p);
-        q = down(q);
-        fx = down(fx);
-        Sx = down(Sx);
-        Sy = down(Sy);
-    }
-    const long long mixed = fix_from<kNodeBits + 2, true>(ac, Ec + 2) - fx;
+    const long long fx = s0 ? dxp1 : -dxm1;
+    const bool wide = ea > E + 2;   // the tail of a front: the diagonal dwarfs the axes
+    if (ea > E + 32) return false;
     if (flat_x || flat_y) {
         const double oc = flat_y ? f(ix, -iy) - (t0 ? ym : yp) : f(-ix, iy) - fy;   // the other quadrant's
-        if ((int)(fix_mag(oc) >> 20) > E + 2) return false;
-        if (mixed != 0 || fix_from<kNodeBits + 2, true>(oc, E + 2) != (flat_y ? fx : -fx)) return false;
+        if (wide || (int)(fix_mag(oc) >> 20) > E + 2) return false;
+        if (fix_from<kNodeBits + 2, true>(ac, E + 2) != fx) return false;
+        if (fix_from<kNodeBits + 2, true>(oc, E + 2) != (flat_y ? fx : -fx)) return false;
     }
-    int L;
+    int L, Ec = E;
     if (time_level == 0 && fix_norm2(p, q, &ps, &qs, &L, &r2)) {
         // (p, q) -= dt/2 Hess grad_(p,q) H, grad H = v0 (p, q) / |(p, q)|
-        const long long cross = (s0 == t0) ? mixed : -mixed;
         const long long y = fix_rsqrt(r2);
         const long long c = fix_mulhi(ps, y, 3), s = fix_mulhi(qs, y, 3);   // the direction, in units of 2^-61
         const long long h = fix_from<kFixBits, true>(vdt, 1023) << 4;   // v0 dt / (2 h) in units of 2^-62
+        const int k = wide ? ea - E - 2 : 0;
+        // the diagonal sets the units of the sums below (the direction kept its own)
+        auto down = [&](long long v) { return (v + ((1ll << k) >> 1)) >> k; };
+        Ec = E + k;
+        const long long mixed = fix_from<kNodeBits + 2, true>(ac, Ec + 2) - (wide ? down(fx) : fx);
+        const long long cross = (s0 == t0) ? mixed : -mixed;
+        if (wide) {
+            p = down(p);
+            q = down(q);
+            Sx = down(Sx);
+            Sy = down(Sy);
+        }
         p -= fix_mulhi(fix_mulhi2(Sx, c, cross, s, 4), h, 2);
         q -= fix_mulhi(fix_mulhi2(cross, c, Sy, s, 4), h, 2);
+        // (|p|, |q| < 2^62.6 for any first differences, diagonal and |v0 dt / h| <= 1)
+        if (wide && (mag(p) | mag(q)) < (1ll << (kNodeBits - 5))) return false;
     }
-    // (|p|, |q| < 2^62.6 for any first differences, diagonal and |v0 dt / h| <= 1)
-    if (wide && (mag(p) | mag(q)) < (1ll << (kNodeBits - 5))) return false;
     double g = 0.0;   // h |grad|
     if (fix_norm2(p, q, &ps, &qs, &L, &r2)) {
         // |(p 2^L, q 2^L)| = 2^61 sqrt(xi), xi = r2 2^-58, sqrt(xi) = xi / sqrt(xi)

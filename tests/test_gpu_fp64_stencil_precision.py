@@ -30,9 +30,9 @@ def _built():
     oracle.set_threads(prev)
 
 
-def one_step(u, theta, v0, level=B.T_MIDPOINT):
+def one_step(u, theta, v0, level=B.T_MIDPOINT, cfl=0.45):
     n2, n1 = u.shape
-    p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=v0, theta=theta, time_level=level, cfl=0.45, autotune=0)
+    p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=v0, theta=theta, time_level=level, cfl=cfl, autotune=0)
     op = oracle.Params(**{k: getattr(p, k) for k in oracle.Params.__dataclass_fields__})
     ref, rc = oracle.run(op, u, 1, K=np.zeros((n2, n1)))   # the prescribed celerity needs no stress
     assert rc == 0
@@ -89,6 +89,24 @@ def test_nodes_beside_a_steep_front(theta, level, v0, n1, n2):
     floor = np.abs(ref - u) < 1e-6
     assert floor.mean() > 0.2
     assert np.linalg.norm((got - ref)[floor]) <= 1e-13 * np.linalg.norm((ref - u)[floor])
+
+
+@pytest.mark.parametrize("e", [2.0 ** -43, 2.0 ** -40, 2.0 ** -30])
+@pytest.mark.parametrize("diagonal", [2.0 ** 20, 2.0 ** 28, 2.0 ** 33])
+@pytest.mark.parametrize("v0", [1.0, -1.0])
+def test_near_tie_beside_a_large_diagonal(e, diagonal, v0):
+    """A node at the bottom of a kink, its one-sided derivatives the differences' own differences of a few e,
+    with diagonals that dwarf them: the gradient's direction comes from the former, its size from the
+    latter.  Every difference is exact in doubles, the increment is three products and a root of
+    them: 1e-14 as above."""
+    u = np.zeros((16, 16))
+    y = x = 8
+    u[y, x + 1], u[y, x - 1], u[y + 1, x], u[y - 1, x] = 1 + 3 * e, 1 + e, 1 + 5 * e, 1 + 2 * e
+    u[y, x + 2] = u[y, x - 2] = u[y + 2, x] = u[y - 2, x] = 9.0
+    u[y + 1, x + 1], u[y - 1, x + 1], u[y + 1, x - 1], u[y - 1, x - 1] = diagonal * 0.5 ** np.arange(4)
+    got, ref = one_step(u, 1.0, v0, cfl=1.0)
+    assert abs(ref[y, x]) > 0.01 * diagonal
+    assert abs(got[y, x] - ref[y, x]) <= 1e-14 * abs(ref[y, x])
 
 
 def annihilation(u, steps, r):
