@@ -316,7 +316,7 @@ FIX_HD void fix_c2r(cfx xk, cfx xc, twx w, cfx* zk, cfx* zc) {
 // twelve and a reciprocal, no speeds and no weights, equal to the whole scheme up to the rounding
 // of its weights' ratio.  The limited second differences make both sides' derivatives agree
 // wherever U13 is smooth, its extrema along the axes included: of the coupled random field 99.7% of
-// the nodes qualify at the start and 98% after 150 steps.  An axis along which nothing varies (both
+// the nodes qualify at the start and 97% after 150 steps.  An axis along which nothing varies (both
 // derivatives, both limited second differences and the cross differences zero) qualifies as well:
 // its two weights of 1/2 belong to equal values.  (FP32: the same skipping took as many instructions
 // as it saved, 69.6 us either way.  Double words: 348 -> 209 us at 2048^2, but a coupled run of 74
@@ -562,7 +562,7 @@ FIX_HD bool fix_upwind(F f, double v0, double dt_h, FixTheta th, int time_level,
     // twice the one-sided derivatives, in half units from here on
     const long long px0 = (dxp1 << 1) - Sx0, px1 = (dxm1 << 1) + Sx1;
     const long long qy0 = (dyp1 << 1) - Sy0, qy1 = (dym1 << 1) + Sy1;
-    // of one sign, and by more than the conversions' rounding (3 at most)
+    // of one sign, and by more than the conversions' rounding (below 4)
     auto mag = [](long long v) { return v ^ (v >> 63); };
     auto one_sign = [&](long long a, long long b) { return (a ^ b) >= 0 && mag(a) >= 8 && mag(b) >= 8; };
     const bool one_x = one_sign(px0, px1), one_y = one_sign(qy0, qy1);
