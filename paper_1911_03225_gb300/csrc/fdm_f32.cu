@@ -7,11 +7,11 @@
 // and the transposition.
 //
 // What bounds them: latency, of global memory at the ends and of the barriers between passes, at
-// 40 to 50 percent of the issue slots.  The arrangement's point is that an access or an index costs
-// no arithmetic of its own: 7.7, 11.0 and 8.3 million warp instructions at 2048^2 (rows forward,
+// 36 to 49 percent of the issue slots.  The arrangement's point is that an access or an index costs
+// no arithmetic of its own: 7.9, 10.1 and 7.9 million warp instructions at 2048^2 (rows forward,
 // columns, rows inverse) against 13.1, 21.3 and 14.5 of the generic kernels.  Measured at 2048^2
-// (bytes read and written at the copy bandwidth: 5, 5 and 8 us): 24.4, 28.3, 29.7 us before, 24.4,
-// 25.4, 22.1 now; at 4096^2 92, 108, 111 before, 71, 68, 75 now.
+// (bytes read and written at the copy bandwidth: 5 us each): 24.4, 28.3, 29.7 us before, 25.6, 24.2,
+// 22.5 now; at 4096^2 92, 108, 111 before, 70, 68, 76 now.
 #include <type_traits>
 
 #include "fdm_fix.cuh"
