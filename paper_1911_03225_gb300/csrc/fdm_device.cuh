@@ -546,7 +546,10 @@ __device__ __forceinline__ void speed_range(double h, double& ap, double& am) {
 // one-sided speeds depend only on the gradient's direction, so they are unchanged; every
 // formula of Steps 1-4 then holds with h = 1 and dt replaced by dt / h.
 // One FP64 node.  The products by theta are skipped or exact where they can be, the weights
-// w(s,t) = nx[s] ny[t] / (dxw dyw) take one reciprocal.
+// w(s,t) = nx[s] ny[t] / (dxw dyw) take one reciprocal.  The scheme squares the differences and is
+// homogeneous in them: where the four to the neighbours lie beyond 2^+-500 it works on 2^-+600 times
+// all of them (exact; not where that would take another one out of range), so it holds up to FP64's
+// ends as fix_upwind does.
 template <typename F>
 __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double theta, int theta_code, int time_level) {
     using T = double;
@@ -559,6 +562,21 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
     // Step 1: first differences and limited second differences along x1 and x2
     T dxm3 = f(-1, 0) - f(-2, 0), dxm1 = f0 - f(-1, 0), dxp1 = f(1, 0) - f0, dxp3 = f(2, 0) - f(1, 0);
     T dym3 = f(0, -1) - f(0, -2), dym1 = f0 - f(0, -1), dyp1 = f(0, 1) - f0, dyp3 = f(0, 2) - f(0, 1);
+    T k = T(1);   // the differences' power of two
+    {
+        auto top = [](unsigned a, unsigned b) { return a > b ? a : b; };
+        auto mag = [](T x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
+        const unsigned m = top(top(mag(dxm1), mag(dxp1)), top(mag(dym1), mag(dyp1)));
+        if (m - (523u << 20) > (1000u << 20)) {
+            const unsigned far = top(top(top(mag(dxm3), mag(dxp3)), top(mag(dym3), mag(dyp3))),
+                                     top(top(mag(f(1, 1) - f(0, 1)), mag(f(-1, 1) - f(0, 1))),
+                                         top(mag(f(1, -1) - f(0, -1)), mag(f(-1, -1) - f(0, -1)))));
+            if (m > (1523u << 20)) k = 0x1p-600;
+            else if (far < (923u << 20)) k = 0x1p600;
+            dxm3 = dxm3 * k; dxm1 = dxm1 * k; dxp1 = dxp1 * k; dxp3 = dxp3 * k;
+            dym3 = dym3 * k; dym1 = dym1 * k; dyp1 = dyp1 * k; dyp3 = dyp3 * k;
+        }
+    }
     Side xs[2], ys[2];  // [0] = + side, [1] = - side
     {
         const T c = theta_mul(dxp1 - dxm1);  // shared by both limiters
@@ -627,7 +645,7 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
         for (int t = 0; t < 2; ++t) {
             const int cy = (t == 0) ? 1 : -1;
             // mixed second difference of the quadrant cell (h^2 times the bilinear cross term)
-            const T mixed = (f(cx, cy) - f(0, cy)) - fx0;
+            const T mixed = (f(cx, cy) - f(0, cy)) * k - fx0;
             const T cross = (cx * cy > 0) ? mixed : -mixed;
             const T val = X + Y[t] + cross * ex * ey[t];   // minus f0, added once below
             T p = dX + cross * ey[t];
@@ -649,7 +667,8 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
         }
         acc += nx[s] * accs;
     }
-    return f0 + acc * inv_w;   // the weights sum to one
+    // the weights sum to one
+    return f0 + acc * (inv_w * (k == T(1) ? T(1) : (k > T(1) ? T(0x1p-600) : T(0x1p600))));
 }
 
 // ---------------------------------------------------------------------------------

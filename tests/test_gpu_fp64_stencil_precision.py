@@ -109,6 +109,23 @@ def test_near_tie_beside_a_large_diagonal(e, diagonal, v0):
     assert abs(got[y, x] - ref[y, x]) <= 1e-14 * abs(ref[y, x])
 
 
+@pytest.mark.parametrize("power", [-990, -940, -700, -520, 520, 700, 1000])
+@pytest.mark.parametrize("theta,level", [(1.0, B.T_MIDPOINT), (1.7, B.T_LITERAL)])
+@pytest.mark.parametrize("n1,n2", [(64, 32), (1024, 256)])
+def test_update_is_homogeneous_to_the_ends_of_the_range(power, theta, level, n1, n2):
+    """Steps 1 to 4 are homogeneous in U13: a step of 2^p U is 2^p times the oracle's step of U, to the
+    rounding of either (1e-14 as above; near the ends a node may take the other form)."""
+    u = np.random.default_rng(14).standard_normal((n2, n1))
+    u[: n2 // 2] += 4.0 * np.sin(2 * np.pi * np.arange(n1) / 16)
+    _, want = one_step(u, theta, 1.0, level)
+    p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=1.0, theta=theta, time_level=level, cfl=0.45, autotune=0)
+    with FDM(p) as sim:
+        sim.set_plastic_distortion(np.ldexp(u, power))
+        sim.step(1)
+        got = np.ldexp(sim.read_fields("up13")["up13"], -power)
+    assert np.linalg.norm(got - want) <= 1e-14 * np.linalg.norm(want - u)
+
+
 def annihilation(u, steps, r):
     """The same scheme on a row that does not vary along x2 (theta = 1, v0 = 1), in the precision of u: the
     x2 weights are halves of equal values, so each side of the x1 axis has one value."""
