@@ -599,9 +599,12 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
     const bool tq = tmag_less(qy[1], qy[0]), tp = tmag_less(px[1], px[0]);
     const T qm = tq ? qy[1] : qy[0], qo = tq ? qy[0] : qy[1];
     const T pm = tp ? px[1] : px[0];
-    auto inv_norm = [&](T p, T q) -> T {   // v0 / |(p, q)|, 0 at the origin
+    // The speeds are kept in units of |v0|: the weights need their ratios alone, and products of
+    // speeds below 2^-511 would not hold them.
+    const unsigned long long vs = ubits(v0) & ~kMagBits;
+    auto inv_norm = [&](T p, T q) -> T {   // sign(v0) / |(p, q)|, 0 at the origin
         const T r2 = p * p + q * q;
-        return tguard(r2) ? v0 * trsqrt(r2) : T(0);
+        return tguard(r2) ? dbits(ubits(trsqrt(r2)) ^ vs) : T(0);
     };
     const T r0 = inv_norm(px[0], qm), r1 = inv_norm(px[1], qm), rc = inv_norm(pm, qo);
     T ap = T(0), am = T(0), bp = T(0), bm = T(0);
@@ -618,6 +621,7 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
     const T inv_w = trcp(dxw * dyw);
     const T vdt = v0 * dt_h;                 // v0 dt / h
     const T hvdt = thalf(vdt);               // v0 dt / (2 h)
+    const T reach = dbits(ubits(vdt) & kMagBits);
     // Step 3: values at the four intermediate points (G2, G3).  Along each direction the
     // limited quadratic on the side's cell, in cell units: with e the displacement / h and
     // sg = -1 on the + side, +1 on the - side,  X(e) = D e + S e (e + sg) / 2 and
@@ -625,7 +629,7 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
     T Y[2], dY[2], ey[2];
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
-        ey[t] = (t == 0 ? bp : bm) * dt_h;
+        ey[t] = (t == 0 ? bp : bm) * reach;
         const T sgn = (t == 0) ? T(-1) : T(1);
         Y[t] = ey[t] * (ys[t].D + thalf(ys[t].S) * (ey[t] + sgn));
         dY[t] = ys[t].D + ys[t].S * (ey[t] + thalf(sgn));
@@ -634,7 +638,7 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         const int cx = (s == 0) ? 1 : -1;
-        const T ex = (s == 0 ? ap : am) * dt_h;
+        const T ex = (s == 0 ? ap : am) * reach;
         const T Dx = xs[s].D, Sx = xs[s].S;
         const T sgn = (s == 0) ? T(-1) : T(1);
         const T X = ex * (Dx + thalf(Sx) * (ex + sgn));
@@ -668,7 +672,7 @@ __device__ __forceinline__ double knp_node(F f, double v0, double dt_h, double t
         acc += nx[s] * accs;
     }
     // the weights sum to one
-    return f0 + acc * (inv_w * (k == T(1) ? T(1) : (k > T(1) ? T(0x1p-600) : T(0x1p600))));
+    return f0 + acc * inv_w * (k == T(1) ? T(1) : (k > T(1) ? T(0x1p-600) : T(0x1p600)));
 }
 
 // ---------------------------------------------------------------------------------

@@ -187,3 +187,19 @@ def test_long_run_does_not_drift():
         gpu += distance(got) ** 2
         cpu += distance(ref.up13) ** 2
     assert gpu ** 0.5 <= 4 * cpu ** 0.5
+
+
+@pytest.mark.parametrize("power", [-620, -520, 400])
+@pytest.mark.parametrize("v0", [1.0, -1.0])
+@pytest.mark.parametrize("n1,n2", [(64, 32), (1024, 256)])
+def test_update_takes_celerities_of_any_size(power, v0, n1, n2):
+    """Under the CFL rule a step depends on the celerity's sign and relative size alone: with 2^p v0 it is
+    the oracle's step with v0, to the rounding of either (1e-14 as above)."""
+    u = np.random.default_rng(15).standard_normal((n2, n1))
+    _, want = one_step(u, 1.7, v0)
+    p = Params(n1=n1, n2=n2, nz=16, nh=4, v0=float(np.ldexp(v0, power)), theta=1.7, cfl=0.45, autotune=0)
+    with FDM(p) as sim:
+        sim.set_plastic_distortion(u)
+        sim.step(1)
+        got = sim.read_fields("up13")["up13"]
+    assert np.linalg.norm(got - want) <= 1e-14 * np.linalg.norm(want - u)
